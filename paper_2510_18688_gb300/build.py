@@ -34,6 +34,7 @@ UNITS = {
     "lbm_api.cu": [],
     "lbm_f32.cu": [],
     "lbm_f64.cu": [],
+    "lbm_node.cu": [],
     "lbm_f16.cu": [],
     "lbm_tan.cu": [],
     "lbm_adjoint.cu": [],

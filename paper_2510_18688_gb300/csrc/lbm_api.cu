@@ -40,6 +40,8 @@ struct lbm_ctx {
   Coef<float> cf;
   Coef<double> cd;
   Coef<lbmk::Dual> ct;   // LBM_FP64_TANGENT: constants with their derivatives
+  lbmn::NodeCoef<double, 2> nd;      // the node step's constants (LBM_FP64)
+  lbmn::NodeCoef<lbmk::Dual, 2> nt;  // and the tangent ones
   bool tangent;          // precision LBM_FP64_TANGENT
   size_t esize;          // bytes per real of the lag fields and phi0
   size_t pop_esize;      // bytes per stored population
@@ -52,8 +54,9 @@ struct lbm_ctx {
   double* staging;       // NFIELD * nx * ny doubles, for host reads (lazy)
   void* in_stage;        // 4 * nx * ny doubles + nx * ny bytes, for host inputs (lazy)
   double* h_diag;        // pinned, NDIAG + 1
-  void* scratch;         // NSCRATCH planes (phi, fs, rho) of the two-kernel step
-  bool split;            // step as macro + collide kernels, or fused (default)
+  bool node;             // steps and read-outs by the node step (double, tangent)
+  bool node0;            // the default of node for this context
+  void* scratch;         // the node step's NSC planes between its two kernels
   int nlag;              // lag planes per buffer: NLAG, plus T for float arithmetic
   // float contexts: the step as the TMA-staged tile kernel (lbm_tile.cuh)
   bool tile;
@@ -217,11 +220,13 @@ void set_tile_config(lbm_ctx* c, int stages, int per_sm) {
   c->tile_grid = per_sm > 0 ? std::max(1, std::min(c->nblocks, per_sm * c->sms)) : c->nblocks;
 }
 
-// Kernel forms of the step (lbm_autotune): 0 one CTA per 32 x 8 tile;
-// 1 float: TMA-staged, one stage, one CTA per tile / FP64: the two-kernel
-// split; 2 TMA-staged, two stages, two persistent CTAs per SM (float);
-// 3 TMA-staged, one stage, three persistent CTAs per SM (float); 4 one CTA
-// per 32 x 4 tile; 5 one CTA per 32 x 16 tile.  Tangent contexts: 0.
+// Kernel forms of the step (lbm_autotune).  Float: 0 one CTA per 32 x 8
+// tile; 1 TMA-staged, one stage, one CTA per tile; 2 TMA-staged, two stages,
+// two persistent CTAs per SM; 3 TMA-staged, one stage, three persistent CTAs
+// per SM; 4 one CTA per 32 x 4 tile; 5 one CTA per 32 x 16 tile.  FP64: 0
+// the node step, on grids of fewer than 32 rows one CTA per 32 x 1 tile; 1
+// the node step; 4 one CTA per 32 x 4 tile; 5 one CTA per 32 x 2 tile.
+// Tangent contexts: 0, the node step.
 bool form_available(const lbm_ctx* c, int form) {
   if (form < 0 || form >= kForms) return false;
   if (c->tangent) return form == 0;
@@ -238,11 +243,12 @@ int tiles_of(const lbm_ctx* c, int ty) {
 void set_kernel_form(lbm_ctx* c, int form) {
   c->form = form;
   c->ty = form == 4 ? 4 : (form == 5 ? 16 : lbmk::TY);
-  if (c->p.precision == LBM_FP64 && !c->tangent) {
-    c->split = form == 1;
+  if (c->tangent) return;
+  if (c->p.precision == LBM_FP64) {
+    c->ty = form == 4 ? 4 : (form == 5 ? 2 : lbmk::THIN_TY);
+    c->node = form == 1 || (form == 0 && c->node0);
     return;
   }
-  c->split = false;
   c->tile = c->tile_ok && form >= 1 && form <= 3;
   if (form == 1) set_tile_config(c, 1, 0);
   else if (form == 2) set_tile_config(c, 2, 2);
@@ -281,18 +287,57 @@ Args<R, S> step_args(lbm_ctx* c, const Coef<R>& coef) {
   return a;
 }
 
+// Warps of a grid of the node step (one set of diagnostic partials each).
+int node_warps(const lbm_ctx* c) { return (c->g.nx * c->g.ny + 31) / 32; }
+
+template <typename R>
+lbmn::NodeArgs<R, 2> node_args(lbm_ctx* c, const lbmn::NodeCoef<R, 2>& coef) {
+  lbmn::NodeArgs<R, 2> a;
+  std::memset((void*)&a, 0, sizeof(a));
+  a.g = lbmh::make_node_geom(c->g);
+  a.c = coef;
+  a.pin = (const R*)c->pop[c->cur];
+  a.pout = (R*)c->pop[c->cur ^ 1];
+  a.lin = (const R*)c->lag[c->cur];
+  a.lout = (R*)c->lag[c->cur ^ 1];
+  a.phi0 = (const R*)c->phi0;
+  a.mask = c->mask;
+  a.sc = (R*)c->scratch;
+  a.diag = c->diag_partial;
+  a.nwarps = node_warps(c);
+  return a;
+}
+
+// One step of a node-step context, or (MODE_READ) the read-out, which leaves
+// the state alone (it writes fl and w into the lag planes the next step will
+// overwrite).
+cudaError_t launch_node_ctx(lbm_ctx* c, int mode, bool diag, double* const* outs, cudaStream_t s) {
+  if (diag) c->diag_nb = node_warps(c);
+  lbmn::ReadOut ro;
+  std::memset(&ro, 0, sizeof(ro));
+  if (outs)
+    for (int k = 0; k < lbmk::NFIELD; k++) ro.out[k] = outs[k];
+  const lbmn::ReadOut* r = mode == lbmk::MODE_READ ? &ro : nullptr;
+  if (c->tangent) return lbmn::launch_node(node_args(c, c->nt), r, diag, s);
+  return lbmn::launch_node(node_args(c, c->nd), r, diag, s);
+}
+
 cudaError_t launch(lbm_ctx* c, int mode, bool diag, double* const* outs, cudaStream_t s) {
+  const bool read = mode == lbmk::MODE_READ;
+  if (read ? c->node0 : c->node) return launch_node_ctx(c, mode, diag, outs, s);
+  if (c->p.precision == LBM_FP64) {
+    const int ty = read ? lbmk::THIN_TY : c->ty;
+    if (diag) c->diag_nb = tiles_of(c, ty);
+    Args<double> a = step_args<double>(c, c->cd);
+    if (outs)
+      for (int k = 0; k < lbmk::NFIELD; k++) a.out[k] = outs[k];
+    return lbmk::launch_step_f64(a, mode, diag, s, ty);
+  }
   // the step launches one CTA per 32 x ty tile (other forms and the
   // read-out: per 32 x 8 tile), each writing one set of diagnostic partials
-  const bool shaped = mode == lbmk::MODE_STEP && !c->split && !c->tile;
+  const bool shaped = mode == lbmk::MODE_STEP && !c->tile;
   const int ty = shaped ? c->ty : lbmk::TY;
   if (diag) c->diag_nb = tiles_of(c, ty);
-  if (mode == lbmk::MODE_STEP && c->split) {  // FP64 only
-    lbmk::SplitArgs<double> a;
-    a.a = step_args<double>(c, c->cd);
-    a.sc = (double*)c->scratch;
-    return lbmk::launch_split_f64(a, diag, s);
-  }
   if (c->p.precision == LBM_FP32) {
     Args<float> a = step_args<float>(c, c->cf);
     if (mode == lbmk::MODE_STEP && c->tile)
@@ -301,25 +346,12 @@ cudaError_t launch(lbm_ctx* c, int mode, bool diag, double* const* outs, cudaStr
       for (int k = 0; k < lbmk::NFIELD; k++) a.out[k] = outs[k];
     return lbmk::launch_step_f32(a, mode, diag, s, ty);
   }
-  if (c->tangent) {
-    Args<lbmk::Dual> a = step_args<lbmk::Dual>(c, c->ct);
-    if (outs)
-      for (int k = 0; k < lbmk::NFIELD; k++) a.out[k] = outs[k];
-    return lbmk::launch_step_tan(a, mode, diag, s);
-  }
-  if (c->p.precision == LBM_FP16S) {
-    Args<float, __half> a = step_args<float, __half>(c, c->cf);
-    if (mode == lbmk::MODE_STEP && c->tile)
-      return lbmk::launch_tile_f16s(tile_args<__half>(c, a), diag, c->tile_stages, c->tile_grid,
-                                    s);
-    if (outs)
-      for (int k = 0; k < lbmk::NFIELD; k++) a.out[k] = outs[k];
-    return lbmk::launch_step_f16s(a, mode, diag, s, ty);
-  }
-  Args<double> a = step_args<double>(c, c->cd);
+  Args<float, __half> a = step_args<float, __half>(c, c->cf);
+  if (mode == lbmk::MODE_STEP && c->tile)
+    return lbmk::launch_tile_f16s(tile_args<__half>(c, a), diag, c->tile_stages, c->tile_grid, s);
   if (outs)
     for (int k = 0; k < lbmk::NFIELD; k++) a.out[k] = outs[k];
-  return lbmk::launch_step_f64(a, mode, diag, s, ty);
+  return lbmk::launch_step_f16s(a, mode, diag, s, ty);
 }
 
 // Steps of one captured period: the buffer parity repeats every two steps
@@ -475,10 +507,10 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
                                                                               : lbmk::NLAG;
   c->g = lbmh::make_geom(*params);
   {
-    // LBM_STEP_KERNEL=split selects the two-kernel step (macro pass +
-    // collide pass); the default is the fused one-kernel step
-    const char* k = std::getenv("LBM_STEP_KERNEL");
-    c->split = k && std::strcmp(k, "split") == 0 && params->precision == LBM_FP64;
+    c->node0 = c->tangent || (params->precision == LBM_FP64 &&
+                              (params->ny >= lbmk::THIN_ROWS ||
+                               (long long)params->nx * params->ny > lbmk::THIN_NODES));
+    c->node = c->node0;
     // LBM_STEP_GRAPHS=0 launches every step on its own instead of
     // replaying captured periods
     const char* gr = std::getenv("LBM_STEP_GRAPHS");
@@ -488,12 +520,20 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
   c->cf = lbmh::make_coef<float>(*params);
   c->cd = lbmh::make_coef<double>(*params);
   if (c->tangent) c->ct = lbmh::make_coef_tangent(*params);
+  const bool f64 = params->precision == LBM_FP64 || c->tangent;
+  if (f64) {
+    const double g[2] = {params->gx, params->gy};
+    c->nd = lbmh::make_node_coef<double, 2>(*params, g, params->T_wall, params->tan_T_wall);
+    c->nt = lbmh::make_node_coef<lbmk::Dual, 2>(*params, g, params->T_wall, params->tan_T_wall);
+  }
   const size_t dmul = c->tangent ? 2 : 1;  // tangent: values, then derivatives
   const dim3 gd = lbmk::grid_dims(c->g);
   c->nblocks = (int)(gd.x * gd.y);
-  c->ty = lbmk::TY;
+  c->ty = f64 ? lbmk::THIN_TY : lbmk::TY;
   c->diag_nb = c->nblocks;
-  c->diag_cap = std::max(c->nblocks, tiles_of(c, 4));  // 32 x 4 tiles write the most
+  // 32 x 4 tiles write the most in float; in double 32 x 1 tiles, of which
+  // there are at least as many as warps of the node step
+  c->diag_cap = tiles_of(c, f64 ? 1 : 4);
   const size_t P = (size_t)c->g.plane;
   cudaError_t e = cudaSuccess;
   for (int b = 0; b < 2 && e == cudaSuccess; b++) {
@@ -501,7 +541,7 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
     if (e == cudaSuccess) e = dev_malloc(&c->lag[b], c->nlag * P * c->esize);
   }
   if (e == cudaSuccess) e = dev_malloc(&c->phi0, P * c->esize);
-  if (e == cudaSuccess) e = dev_malloc(&c->scratch, lbmk::NSCRATCH * P * c->esize);
+  if (e == cudaSuccess && f64) e = dev_malloc(&c->scratch, lbmn::NSC * P * c->esize);
   if (e == cudaSuccess) e = dev_malloc((void**)&c->mask, P);
   if (e == cudaSuccess)
     e = dev_malloc((void**)&c->diag_partial, dmul * lbmk::NDIAG * c->diag_cap * sizeof(double));
@@ -1767,10 +1807,15 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, void* stream, doubl
 struct lbm_batch {
   std::vector<lbm_ctx*> ctx;
   int precision;
-  // FP32 batches step as the batched TMA-staged tile kernel (one stage, one
-  // CTA per tile) unless LBM_BATCH_KERNEL=fused; its argument table
-  bool tile;
+  // argument tables of the batch's kernels: FP64 the node step and, for grids
+  // of few rows, one CTA per 32 x 1 tile (the contexts of each in `nodes` and
+  // `thin`); FP32 the batched TMA-staged tile kernel (one stage, one CTA per
+  // tile) or, with LBM_BATCH_KERNEL=fused, one CTA per tile from global memory
+  std::vector<lbm_ctx*> nodes, thin;
+  lbmn::NodeBatch* ntab;
+  lbmk::BatchTable<double>* dtab;
   lbmk::TileBatch<float>* ttab;
+  lbmk::BatchTable<float>* ftab;
   cudaStream_t cap_stream;
   cudaGraphExec_t graph;               // one captured period of batch steps
   std::vector<uint64_t> graph_key;     // (parity, generation) per context, phase
@@ -1779,33 +1824,46 @@ struct lbm_batch {
 
 namespace {
 
-// One launch covers up to BATCH_MAX_GRIDS consecutive contexts; the table
-// holds each one's step arguments (buffers by its current parity).
+// One launch covers up to BATCH_MAX_GRIDS consecutive contexts of a list; the
+// table holds each one's step arguments (buffers by its current parity).
 template <typename R>
-bool fill_table(lbm_batch* b, int first, int count, lbmk::BatchTable<R>& t) {
+bool fill_table(lbm_ctx* const* ctx, int count, lbmk::BatchTable<R>& t, int ty) {
   bool all = true;
   t.ngrids = count;
   t.tile_base[0] = 0;
   for (int i = 0; i < count; i++) {
-    lbm_ctx* c = b->ctx[first + i];
-    const Coef<R>* coef;
-    if (sizeof(R) == 4) coef = (const Coef<R>*)(const void*)&c->cf;
-    else coef = (const Coef<R>*)(const void*)&c->cd;
-    t.args[i] = step_args<R>(c, *coef);
-    t.tile_base[i + 1] = t.tile_base[i] + c->nblocks;
+    lbm_ctx* c = ctx[i];
+    if constexpr (sizeof(R) == 4) t.args[i] = step_args<float>(c, c->cf);
+    else t.args[i] = step_args<double>(c, c->cd);
+    t.tile_base[i + 1] = t.tile_base[i] + tiles_of(c, ty);
     if (c->p.lattices != 7u) all = false;
   }
   return all;
 }
 
-// The batched tile kernel's table for contexts [first, first + count).
-bool fill_tile_table(lbm_batch* b, int first, int count, lbmk::TileBatch<float>& t) {
+// The node step's table.
+bool fill_node_table(lbm_ctx* const* ctx, int count, lbmn::NodeBatch& t) {
+  bool all = true;
+  t.ngrids = count;
+  t.base[0] = 0;
+  for (int i = 0; i < count; i++) {
+    lbm_ctx* c = ctx[i];
+    t.args[i] = node_args(c, c->nd);
+    t.base[i + 1] = t.base[i] + (t.args[i].g.nodes + lbmn::NODE_BATCH_THREADS - 1) /
+                                    lbmn::NODE_BATCH_THREADS;
+    if (c->p.lattices != 7u) all = false;
+  }
+  return all;
+}
+
+// The batched tile kernel's table.
+bool fill_tile_table(lbm_ctx* const* ctx, int count, lbmk::TileBatch<float>& t) {
   bool all = true;
   t.ngrids = count;
   t.tile_base[0] = 0;
   t.extra_tx = g_tile_timeout.load() ? 16u : 0u;
   for (int i = 0; i < count; i++) {
-    lbm_ctx* c = b->ctx[first + i];
+    lbm_ctx* c = ctx[i];
     t.args[i] = step_args<float>(c, c->cf);
     t.tile_base[i + 1] = t.tile_base[i] + c->nblocks;
     t.tiles_x[i] = (c->g.nx + lbmk::TX - 1) / lbmk::TX;
@@ -1828,35 +1886,55 @@ void note_batch_diag(lbm_batch* b, int64_t first0, int64_t n) {
   for (lbm_ctx* c : b->ctx) {
     c->have_diag = true;
     c->diag_pending = true;
-    c->diag_nb = c->nblocks;  // the batch kernel's 32 x 8 tiles
+    // the batch kernels' partials: a set per warp, 32 x 1 or 32 x 8 tile
+    c->diag_nb = c->p.precision != LBM_FP64 ? c->nblocks
+                 : c->node0                 ? node_warps(c)
+                                            : tiles_of(c, lbmk::THIN_TY);
     c->diag_step = c->step + (last - first0);
   }
 }
 
-template <typename R>
-cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s,
-                           lbmk::BatchTable<R>& t) {
-  const int n = (int)b->ctx.size();
+// One step of a list of contexts by the kernel `kind` of their group.
+enum { BATCH_NODE, BATCH_THIN, BATCH_TILE, BATCH_FUSED };
+cudaError_t batch_group(lbm_batch* b, const std::vector<lbm_ctx*>& list, int kind, bool diag,
+                        cudaStream_t s) {
+  static_assert(lbmn::NODE_BATCH_GRIDS == lbmk::BATCH_MAX_GRIDS, "one chunk size for all tables");
+  const int n = (int)list.size();
+  for (int first = 0; first < n; first += lbmk::BATCH_MAX_GRIDS) {
+    const int count = std::min(n - first, lbmk::BATCH_MAX_GRIDS);
+    lbm_ctx* const* ctx = list.data() + first;
+    cudaError_t e;
+    if (kind == BATCH_NODE) {
+      const bool all = fill_node_table(ctx, count, *b->ntab);
+      e = lbmn::launch_node_batch(*b->ntab, diag, all, s);
+    } else if (kind == BATCH_THIN) {
+      const bool all = fill_table(ctx, count, *b->dtab, lbmk::THIN_TY);
+      e = lbmk::launch_batch_f64(*b->dtab, diag, all, s);
+    } else if (kind == BATCH_TILE) {
+      const bool all = fill_tile_table(ctx, count, *b->ttab);
+      e = lbmk::launch_tile_batch_f32(*b->ttab, diag, all, s);
+    } else {
+      const bool all = fill_table(ctx, count, *b->ftab, lbmk::TY);
+      e = lbmk::launch_batch_f32(*b->ftab, diag, all, s);
+    }
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
   lbm_ctx* c0 = b->ctx[0];
   for (int64_t k = 0; k < nsteps; k++) {
     const bool diag = c0->p.diag_every > 0 && (c0->step % c0->p.diag_every) == 0;
-    for (int first = 0; first < n; first += lbmk::BATCH_MAX_GRIDS) {
-      const int count = std::min(n - first, lbmk::BATCH_MAX_GRIDS);
-      cudaError_t e;
-      if (sizeof(R) == 4 && b->tile) {
-        const bool all = fill_tile_table(b, first, count, *b->ttab);
-        e = lbmk::launch_tile_batch_f32(*b->ttab, diag, all, s);
-        if (e != cudaSuccess) return e;
-        continue;
-      }
-      const bool all = fill_table<R>(b, first, count, t);
-      if (sizeof(R) == 4)
-        e = lbmk::launch_batch_f32(*(const lbmk::BatchTable<float>*)(const void*)&t, diag, all, s);
-      else
-        e = lbmk::launch_batch_f64(*(const lbmk::BatchTable<double>*)(const void*)&t, diag, all,
-                                   s);
-      if (e != cudaSuccess) return e;
+    cudaError_t e;
+    if (b->precision == LBM_FP64) {
+      // each grid by its own default kernel, as lbm_step takes it
+      e = batch_group(b, b->nodes, BATCH_NODE, diag, s);
+      if (e == cudaSuccess) e = batch_group(b, b->thin, BATCH_THIN, diag, s);
+    } else {
+      e = batch_group(b, b->ctx, b->ttab ? BATCH_TILE : BATCH_FUSED, diag, s);
     }
+    if (e != cudaSuccess) return e;
     note_batch_diag(b, c0->step, 1);
     for (lbm_ctx* c : b->ctx) {
       c->cur ^= 1;
@@ -1880,8 +1958,7 @@ std::vector<uint64_t> batch_key(const lbm_batch* b, int period) {
 
 // The captured period of batch steps from the contexts' current parities
 // and phase (captured on a private stream when first needed).
-template <typename R>
-cudaError_t batch_graph(lbm_batch* b, int period, lbmk::BatchTable<R>& t, cudaGraphExec_t* out) {
+cudaError_t batch_graph(lbm_batch* b, int period, cudaGraphExec_t* out) {
   std::vector<uint64_t> key = batch_key(b, period);
   if (b->graph && key == b->graph_key) {
     *out = b->graph;
@@ -1904,7 +1981,7 @@ cudaError_t batch_graph(lbm_batch* b, int period, lbmk::BatchTable<R>& t, cudaGr
     saved.push_back({c->cur, c->step, c->diag_step, c->have_diag, c->diag_pending});
   e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  cudaError_t el = batch_launches<R>(b, period, b->cap_stream, t);
+  cudaError_t el = batch_launches(b, period, b->cap_stream);
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(b->cap_stream, &g);
   for (size_t i = 0; i < b->ctx.size(); i++) {
@@ -1930,17 +2007,14 @@ cudaError_t batch_graph(lbm_batch* b, int period, lbmk::BatchTable<R>& t, cudaGr
   return cudaSuccess;
 }
 
-template <typename R>
 int batch_step_impl(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
-  std::unique_ptr<lbmk::BatchTable<R>> t(new (std::nothrow) lbmk::BatchTable<R>());
-  if (!t) return LBM_ERR_OOM;
   lbm_ctx* c0 = b->ctx[0];
   int64_t left = nsteps;
   const int period = graph_period(c0->p.diag_every, c0->graph_min);
   cudaError_t e = cudaSuccess;
   if (c0->graphs && period <= kMaxGraphSteps && left >= period && stream_free(s)) {
     cudaGraphExec_t g = nullptr;
-    e = batch_graph<R>(b, period, *t, &g);
+    e = batch_graph(b, period, &g);
     if (e != cudaSuccess) {
       std::snprintf(b->err, sizeof(b->err), "batch graph capture: %s", cudaGetErrorString(e));
       return LBM_ERR_CUDA;
@@ -1955,7 +2029,7 @@ int batch_step_impl(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
     for (lbm_ctx* c : b->ctx) c->step += reps * period;  // even period: parities unchanged
     left -= reps * period;
   }
-  e = batch_launches<R>(b, left, s, *t);
+  e = batch_launches(b, left, s);
   for (lbm_ctx* c : b->ctx) c->last_stream = s;
   if (e != cudaSuccess) {
     std::snprintf(b->err, sizeof(b->err), "batch kernel launch: %s", cudaGetErrorString(e));
@@ -1982,16 +2056,21 @@ int lbm_batch_create(lbm_ctx* const* ctxs, int count, lbm_batch** out) {
   if (!b) return LBM_ERR_OOM;
   b->ctx.assign(ctxs, ctxs + count);
   b->precision = ctxs[0]->p.precision;
-  b->tile = b->precision == LBM_FP32;
-  for (int i = 0; i < count; i++) b->tile = b->tile && ctxs[i]->tile_ok && ctxs[i]->d_maps;
-  if (const char* k = std::getenv("LBM_BATCH_KERNEL"))
-    if (std::strcmp(k, "fused") == 0) b->tile = false;
-  if (b->tile) {
-    b->ttab = new (std::nothrow) lbmk::TileBatch<float>();
-    if (!b->ttab) {
-      delete b;
-      return LBM_ERR_OOM;
-    }
+  if (b->precision == LBM_FP64) {
+    for (lbm_ctx* c : b->ctx) (c->node0 ? b->nodes : b->thin).push_back(c);
+    b->ntab = new (std::nothrow) lbmn::NodeBatch();
+    b->dtab = new (std::nothrow) lbmk::BatchTable<double>();
+  } else {
+    bool tile = true;
+    for (int i = 0; i < count; i++) tile = tile && ctxs[i]->tile_ok && ctxs[i]->d_maps;
+    if (const char* k = std::getenv("LBM_BATCH_KERNEL"))
+      if (std::strcmp(k, "fused") == 0) tile = false;
+    if (tile) b->ttab = new (std::nothrow) lbmk::TileBatch<float>();
+    else b->ftab = new (std::nothrow) lbmk::BatchTable<float>();
+  }
+  if (b->precision == LBM_FP64 ? !(b->ntab && b->dtab) : !(b->ttab || b->ftab)) {
+    lbm_batch_destroy(b);
+    return LBM_ERR_OOM;
   }
   *out = b;
   return LBM_OK;
@@ -2009,15 +2088,17 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps, void* stream) {
   }
   if (nsteps == 0) return LBM_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  return b->precision == LBM_FP32 ? batch_step_impl<float>(b, nsteps, s)
-                                  : batch_step_impl<double>(b, nsteps, s);
+  return batch_step_impl(b, nsteps, s);
 }
 
 void lbm_batch_destroy(lbm_batch* b) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+  delete b->ntab;
+  delete b->dtab;
   delete b->ttab;
+  delete b->ftab;
   delete b;
 }
 

@@ -1,10 +1,11 @@
-// lbm_f64.cu -- instantiation of the fused step, read-out and init kernels
-// for double arithmetic (sm_103a).
+// lbm_f64.cu -- double-precision kernels beside the node step (sm_103a): the
+// initial state, the diagnostics of a caller-held state, crossings, and the
+// sum of the diagnostic partials.
 #include "lbm_launch.h"
 
 namespace lbmk {
 
-template <int MODE, bool DIAG, int TYS = TY>
+template <int MODE, bool DIAG, int TYS>
 static void launch_one(const Args<double>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
@@ -16,9 +17,9 @@ static void launch_one(const Args<double>& a, cudaStream_t s) {
 
 template <bool DIAG>
 static void launch_shape(const Args<double>& a, int ty, cudaStream_t s) {
-  if (ty == 4) launch_one<MODE_STEP, DIAG, 4>(a, s);
-  else if (ty == 16) launch_one<MODE_STEP, DIAG, 16>(a, s);
-  else launch_one<MODE_STEP, DIAG>(a, s);
+  if (ty == 1) launch_one<MODE_STEP, DIAG, 1>(a, s);
+  else if (ty == 2) launch_one<MODE_STEP, DIAG, 2>(a, s);
+  else launch_one<MODE_STEP, DIAG, 4>(a, s);
 }
 
 cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s, int ty) {
@@ -26,37 +27,27 @@ cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStre
     if (diag) launch_shape<true>(a, ty, s);
     else launch_shape<false>(a, ty, s);
   } else {
-    if (diag) launch_one<MODE_READ, true>(a, s);
-    else launch_one<MODE_READ, false>(a, s);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_split_f64(const SplitArgs<double>& a, bool diag, cudaStream_t s) {
-  const dim3 grid = grid_dims(a.a.g), block = block_dims();
-  const bool all = a.a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT);
-  if (all) lbm_macro_kernel<double, 7><<<grid, block, 0, s>>>(a);
-  else lbm_macro_kernel<double, 0><<<grid, block, 0, s>>>(a);
-  if (all) {
-    if (diag) lbm_collide_kernel<double, true, 7><<<grid, block, 0, s>>>(a);
-    else lbm_collide_kernel<double, false, 7><<<grid, block, 0, s>>>(a);
-  } else {
-    if (diag) lbm_collide_kernel<double, true, 0><<<grid, block, 0, s>>>(a);
-    else lbm_collide_kernel<double, false, 0><<<grid, block, 0, s>>>(a);
+    if (diag) launch_one<MODE_READ, true, THIN_TY>(a, s);
+    else launch_one<MODE_READ, false, THIN_TY>(a, s);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s) {
-  const dim3 block = block_dims();
+  const dim3 block = block_dims(THIN_TY);
   const int ctas = b.tile_base[b.ngrids];
   if (all) {
-    if (diag) lbm_batch_kernel<double, true, 7><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<double, false, 7><<<ctas, block, 0, s>>>(b);
+    if (diag) lbm_batch_kernel<double, true, 7, THIN_TY><<<ctas, block, 0, s>>>(b);
+    else lbm_batch_kernel<double, false, 7, THIN_TY><<<ctas, block, 0, s>>>(b);
   } else {
-    if (diag) lbm_batch_kernel<double, true, 0><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<double, false, 0><<<ctas, block, 0, s>>>(b);
+    if (diag) lbm_batch_kernel<double, true, 0, THIN_TY><<<ctas, block, 0, s>>>(b);
+    else lbm_batch_kernel<double, false, 0, THIN_TY><<<ctas, block, 0, s>>>(b);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_diag_f64(const Args<double>& a, cudaStream_t s) {
+  lbm_step_kernel<double, MODE_READ, true, 0><<<grid_dims(a.g), block_dims(), 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -154,7 +145,7 @@ cudaError_t launch_init_f64(const InitArgs<double>& a, cudaStream_t s) {
 
 cudaError_t launch_diag_finalize(const double* partial, int nb, double* out, long long step,
                                  cudaStream_t s) {
-  lbm_diag_finalize_kernel<<<1, NT, 0, s>>>(partial, nb, out, step);
+  lbm_diag_finalize_kernel<<<NDIAG, NT, 0, s>>>(partial, nb, out, step);
   return cudaGetLastError();
 }
 

@@ -8,6 +8,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_kernels.cuh"
+#include "lbm_node.cuh"
 
 namespace lbmh {
 
@@ -72,6 +73,76 @@ inline Coef<lbmk::Dual> make_coef_tangent(const lbm_params& p) {
   c.cos_th.d = -std::sin(p.theta_deg * pi / 180.0) * (pi / 180.0) * p.tan_theta_deg;
   c.latent.d = p.tan_latent;
   return c;
+}
+
+// A constant of the step with (tangent) or without its derivative.
+template <typename R>
+R directed(double v, double d) {
+  if constexpr (lbmk::is_dual<R>::value) return R(v, d);
+  else { (void)d; return (R)v; }
+}
+
+// Constants of the node step; g: the D body-force components, T, dT: the 2 D
+// wall temperatures and their rates along the parameter direction.
+template <typename R, int D>
+inline lbmn::NodeCoef<R, D> make_node_coef(const lbm_params& p, const double* g, const double* T,
+                                           const double* dT) {
+  using k_t = lbmn::K<R>;
+  lbmn::NodeCoef<R, D> c;
+  const double deg = 3.14159265358979323846 / 180.0;
+  const double pr[4][3] = {{p.rho_s, p.rho_l, p.rho_g}, {p.mu_s, p.mu_l, p.mu_g},
+                           {p.lambda_s, p.lambda_l, p.lambda_g}, {p.cp_s, p.cp_l, p.cp_g}};
+  for (int k = 0; k < 3; k++) {
+    c.rho[k] = (k_t)pr[0][k];
+    c.mu[k] = (k_t)pr[1][k];
+    c.lam[k] = (k_t)pr[2][k];
+    c.cp[k] = (k_t)pr[3][k];
+  }
+  // Cp_ref = 2 Cp_s Cp_l / (Cp_s + Cp_l) (Sec. 3.3)
+  const double rr = p.rho_ref * (2.0 * p.cp_s * p.cp_l / (p.cp_s + p.cp_l));
+  c.rr = (k_t)rr;
+  c.inv_rr3 = (k_t)(3.0 / rr);
+  const double s3 = 3.0 * p.sigma / p.eps;
+  const double ct = std::cos(p.theta_deg * deg), cp = std::cos(p.psi_deg * deg);
+  const double dct = -std::sin(p.theta_deg * deg) * deg * p.tan_theta_deg;
+  c.s3 = (k_t)s3;
+  c.s9 = (k_t)(9.0 * p.sigma / p.eps);
+  c.klap = (k_t)(3.0 * p.eps * p.sigma / 8.0);
+  c.s3cp = (k_t)(s3 * cp);
+  c.cos_ps = (k_t)cp;
+  c.cos_th = directed<R>(ct, dct);
+  c.s3ct = directed<R>(s3 * ct, s3 * dct);
+  const double itg = 1.0 / (0.5 + p.mobility / (p.eta / 3.0));  // Eq. (21)
+  const double gc = 1.0 - 0.5 * itg, w1 = lbmn::Lat<D>::w1;
+  c.itg = (k_t)itg;
+  c.eta = (k_t)p.eta;
+  c.omg = (k_t)(1.0 - itg);
+  c.itg_eta = (k_t)(itg * p.eta);
+  c.gcoef = (k_t)gc;
+  c.v_new = (k_t)(3.0 * w1 * (itg + gc));
+  c.v_old = (k_t)(3.0 * w1 * gc);
+  c.ratio = (k_t)(1.0 - p.rho_s / p.rho_l);
+  for (int k = 0; k < D; k++) c.g[k] = (k_t)g[k];
+  c.rl = directed<R>(p.rho_l * p.latent, p.rho_l * p.tan_latent);
+  c.T_cold = directed<R>(p.T_cold, p.tan_T_cold);
+  for (int k = 0; k < 2 * D; k++) c.T_wall[k] = directed<R>(T[k], dT[k]);
+  c.readings = p.readings;
+  return c;
+}
+
+inline lbmn::NodeGeom<2> make_node_geom(const Geom& g) {
+  lbmn::NodeGeom<2> q;
+  q.n[0] = g.nx;
+  q.n[1] = g.ny;
+  q.pitch = g.pitch;
+  q.nodes = g.nx * g.ny;
+  q.dx = lbmn::make_fastdiv((unsigned)g.nx);
+  q.dy = lbmn::make_fastdiv((unsigned)g.ny);
+  q.plane = g.plane;
+  for (int k = 0; k < 4; k++) q.bc[k] = g.bc[k];
+  q.lattices = g.lattices;
+  q.has_mask = g.has_mask;
+  return q;
 }
 
 inline int validate(const lbm_params* p, char* err, size_t n) {

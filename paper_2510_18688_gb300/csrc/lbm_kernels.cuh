@@ -52,7 +52,7 @@ static_assert(RING * NPART <= NT, "ring loads must fit one pass of the CTA");
 // nodes per 256 at 32 x 8, 100 per 512 at 32 x 16).
 template <int TY_>
 struct Shape {
-  static_assert(TY_ == 4 || TY_ == 8 || TY_ == 16, "tile shapes 32 x 4, 32 x 8, 32 x 16");
+  static_assert(TY_ == 1 || TY_ == 2 || TY_ == 4 || TY_ == 8 || TY_ == 16, "a divisor or multiple of 8");
   static constexpr int TY = TY_, HY = TY_ + 2, HN = HX * HY, NT = TX * TY_, RING = HN - NT;
 };
 __host__ __device__ constexpr int tiles_y(int ny, int ty) { return (ny + ty - 1) / ty; }
@@ -656,35 +656,32 @@ __device__ __forceinline__ void block_diag(const R* dvals, R (*s_red)[NDIAG],
              gridDim.x * gridDim.y);
 }
 
-// Grid-wide FP64 diagnostics from the per-CTA partials, one CTA, fixed order
-// (bitwise reproducible): out[0..NDIAG-1] = sums, out[NDIAG] = step index.
-static __global__ void __launch_bounds__(NT) lbm_diag_finalize_kernel(const double* __restrict__ partial,
-                                                               int nb, double* __restrict__ out,
-                                                               long long step) {
-  __shared__ double s_red[NT / 32][NDIAG];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double acc[NDIAG];
+// Grid-wide FP64 diagnostics from the partial sums (nb per diagnostic, one
+// per CTA or warp of the step): CTA k sums row k in a fixed order (bitwise
+// reproducible); out[0..NDIAG-1] = sums, out[NDIAG] = step index.
+static __global__ void __launch_bounds__(NT) lbm_diag_finalize_kernel(
+    const double* __restrict__ partial, int nb, double* __restrict__ out, long long step) {
+  __shared__ double s_red[NT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = blockIdx.x;
+  const double* row = partial + (long long)k * nb;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};  // four loads in flight
+  for (int j = tid; j < nb; j += 4 * NT) {
 #pragma unroll
-  for (int k = 0; k < NDIAG; k++) acc[k] = 0.0;
-  for (int j = tid; j < nb; j += NT) {
-#pragma unroll
-    for (int k = 0; k < NDIAG; k++) acc[k] += partial[(long long)k * nb + j];
+    for (int q = 0; q < 4; q++)
+      if (j + q * NT < nb) acc[q] += row[j + q * NT];
   }
+  double v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
-  for (int k = 0; k < NDIAG; k++) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) s_red[warp][k] = v;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s_red[warp] = v;
   __syncthreads();
-  if (tid < NDIAG) {
+  if (tid == 0) {
     double t = 0.0;
 #pragma unroll
-    for (int w = 0; w < NT / 32; w++) t += s_red[w][tid];
-    out[tid] = t;
+    for (int w = 0; w < NT / 32; w++) t += s_red[w];
+    out[k] = t;
+    if (k == 0) out[NDIAG] = (double)step;
   }
-  if (tid == 0) out[NDIAG] = (double)step;
 }
 
 // ---------------------------------------------------------------------------

@@ -6,7 +6,7 @@
 
 #include "lbm_kernels.cuh"
 #include "lbm_step.cuh"
-#include "lbm_split.cuh"
+#include "lbm_node.cuh"
 #include "lbm_tile.cuh"
 
 namespace lbmk {
@@ -20,10 +20,21 @@ inline dim3 grid_dims(const Geom& g, int ty = TY) {
 // on 32 x ty tiles (ty = 4, 8 or 16), MODE_READ on 32 x 8.
 cudaError_t launch_step_f32(const Args<float>& a, int mode, bool diag, cudaStream_t s,
                             int ty = TY);
-cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s,
-                            int ty = TY);
-// Two-kernel form of MODE_STEP (macro pass, then collide pass).
-cudaError_t launch_split_f64(const SplitArgs<double>& a, bool diag, cudaStream_t s);
+// Double on grids of fewer than THIN_ROWS rows and at most THIN_NODES nodes
+// -- the one-dimensional columns -- stays with the fused tile: MODE_STEP on
+// 32 x ty tiles (ty = 1, 2 or 4), MODE_READ and batches on 32 x THIN_TY.  The
+// node step is the faster one there too (512 x 8: 14.6 us a step; fused 57 us
+// on 32 x 8 tiles, 42 us on 32 x 1), but across a column the velocity is
+// nothing but rounding (1e-20 against 4e-5 along it), and the fused tile
+// keeps every bit of it as earlier results and saved runs have it.  One warp
+// a tile spreads a column over the most SMs; with it the step is a single
+// warp's chain of FP64 latencies whatever the size up to the bound.
+constexpr int THIN_ROWS = 32, THIN_NODES = 32768, THIN_TY = 1;
+cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s, int ty);
+cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s);
+// The diagnostics of a caller-held double state, which has no room for the
+// node step's planes.
+cudaError_t launch_diag_f64(const Args<double>& a, cudaStream_t s);
 cudaError_t launch_init_f32(const InitArgs<float>& a, cudaStream_t s);
 // The float step as the TMA-staged tile kernel (lbm_tile.cuh) with 1 or 2
 // shared-memory stages on `grid` CTAs (persistent when grid < tiles);
@@ -50,12 +61,10 @@ cudaError_t launch_adjoint_step(const AdjArgs& a, cudaStream_t s);
 cudaError_t launch_adjoint_init(const AdjArgs& a, cudaStream_t s);
 cudaError_t launch_adjoint_reduce(const double* acc, const Geom& g, double* out, cudaStream_t s);
 // Forward-mode tangent (FP64 value and derivative).
-cudaError_t launch_step_tan(const Args<Dual>& a, int mode, bool diag, cudaStream_t s);
 cudaError_t launch_init_tan(const InitArgs<Dual>& a, cudaStream_t s);
 // Up to BATCH_MAX_GRIDS grids in one launch, one CTA per tile.
 cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, cudaStream_t s);
-cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s);
-// Grid-wide diagnostics from the per-CTA partials (one CTA).
+// Grid-wide diagnostics from the partial sums (one CTA per diagnostic).
 cudaError_t launch_diag_finalize(const double* partial, int nb, double* out, long long step,
                                  cudaStream_t s);
 cudaError_t launch_init_f64(const InitArgs<double>& a, cudaStream_t s);
@@ -66,3 +75,15 @@ cudaError_t launch_crossings(const double* phi, const double* w, const double* f
                              int ny, int axis, int index, double* out, cudaStream_t s);
 
 }  // namespace lbmk
+
+namespace lbmn {
+
+// The node step (double, Dual): one time step, or with ro the read-out of the
+// state's fields.
+template <typename R>
+cudaError_t launch_node(const NodeArgs<R, 2>& a, const ReadOut* ro, bool diag,
+                        cudaStream_t s);
+// Up to NODE_BATCH_GRIDS double grids in one pair of launches.
+cudaError_t launch_node_batch(const NodeBatch& b, bool diag, bool all, cudaStream_t s);
+
+}  // namespace lbmn

@@ -113,7 +113,7 @@ extern "C" int lbm_diagnostics_noalloc(const lbm_params* params, const void* pop
       a.phi0 = (const double*)phi0;
       a.mask = cold_mask;
       a.diag_partial = scratch;
-      e = lbmk::launch_step_f64(a, lbmk::MODE_READ, true, s);
+      e = lbmk::launch_diag_f64(a, s);
     }
   }
   if (e == cudaSuccess) e = lbmk::launch_diag_finalize(scratch, (int)nb, out, 0, s);

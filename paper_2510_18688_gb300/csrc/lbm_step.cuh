@@ -708,8 +708,7 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
   __syncthreads();
 
   // ---- phase A2: inversion, order parameter, properties of the ring ---------
-  if (tid < RING) {
-    const int k = tid;
+  auto ring_state = [&](int k) {
     int hx, hy;
     ring_pos<TYS>(k, hx, hy);
     const int hi = hy * HX + hx;
@@ -743,6 +742,11 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     s_fs[hi] = Lq.fs;
     s_rho[hi] = Lq.rho;
     if constexpr (WB) s_T[hi] = Lq.T;
+  };
+  if constexpr (RING <= NT) {
+    if (tid < RING) ring_state(tid);
+  } else {
+    for (int k = tid; k < RING; k += NT) ring_state(k);
   }
   __syncthreads();
 
@@ -858,7 +862,12 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     }
   }
   };
-  if (x0 >= 1 && x0 + TX < g.nx && y0 >= 1 && y0 + TY < g.ny) phase_b(std::true_type{});
+  // short tiles take the path of the 32 x 8 tile they are part of: the two
+  // copies of the arithmetic may round differently, so a node's last bits do
+  // not depend on the tile height
+  constexpr int TYB = TY < 8 ? 8 : TY;
+  const int yb = y0 / TYB * TYB;
+  if (x0 >= 1 && x0 + TX < g.nx && yb >= 1 && yb + TYB < g.ny) phase_b(std::true_type{});
   else phase_b(std::false_type{});
   if (DIAG) {
     if (b < 0)
@@ -893,8 +902,8 @@ struct BatchTable {
   Args<R> args[BATCH_MAX_GRIDS];
 };
 
-template <typename R, bool DIAG, int LATC>
-__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
+template <typename R, bool DIAG, int LATC, int TYS = TY>
+__global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
     lbm_batch_kernel(const __grid_constant__ BatchTable<R> B) {
   const int t = blockIdx.x;
   int lo = 0, hi = B.ngrids;  // tile_base[lo] <= t < tile_base[hi]
@@ -907,7 +916,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
   const int local = t - B.tile_base[lo];
   const int tiles_x = (a.g.nx + TX - 1) / TX;
   const int ntiles = B.tile_base[lo + 1] - B.tile_base[lo];
-  step_tile<R, MODE_STEP, DIAG, LATC>(a, local % tiles_x, local / tiles_x, local, ntiles);
+  step_tile<R, MODE_STEP, DIAG, LATC, R, TYS>(a, local % tiles_x, local / tiles_x, local, ntiles);
 }
 
 }  // namespace lbmk

@@ -1,0 +1,137 @@
+"""The double-precision node step: grids at the edges of its warps, blocks and
+of the rule that leaves grids of few rows to the fused tile; batches that mix
+the two; the reciprocal its kernels take."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from paper_2510_18688_gb300 import workloads as W
+
+FIELDS = ("phi", "fs", "fl", "T", "rhoH", "p", "ux", "uy", "rho", "mu", "w", "mdot")
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from oracle import oracle as O
+    from paper_2510_18688_gb300 import build, lbm
+    build.build()
+    lbm.load()
+    return O, lbm
+
+
+def _close(got, ref, tol=1e-10):  # the parity bar of the FP64 step
+    for k in FIELDS:
+        scale = max(np.abs(ref[k]).max(), 1e-300)
+        assert np.abs(got[k] - ref[k]).max() <= tol * scale + 1e-18, k
+
+
+# columns of one warp and less, rows that end inside a warp and a block, one
+# row to each side of the rule's 32 rows, and of its 32768 nodes
+SIZES = [(2, 32), (3, 33), (31, 32), (32, 32), (33, 32), (33, 31), (64, 64), (129, 33), (40, 200),
+         (1057, 31), (1060, 31), (701, 39)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("seed", [0, 3])
+def test_sizes_match_the_oracle(env, nx, ny, seed):
+    O, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=seed)
+    steps = 21
+    o = O.from_workload((cfg, arr)).step(steps - 1)
+    rd = o.diagnostics()
+    s = lbm.Solver(cfg, precision="fp64", diag_every=1).set_geometry(arr).step(steps)
+    d = s.diagnostics(compute=False)
+    _close(s.fields(), o.step(1).fields())
+    for k, v in rd.items():
+        if k != "step":
+            assert abs(d[k] - v) <= 1e-12 * (abs(v) + nx * ny), k
+    s.close()
+
+
+# (grids of fewer rows take the fused tile, whose copies with and without sums
+# round some nodes differently)
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [z for z in SIZES if z[1] >= 32])
+@pytest.mark.parametrize("seed", [0, 3])
+def test_fused_sums_equal_the_read_out(env, nx, ny, seed):
+    """The read-out's sums of a state are those fused into the step that read
+    it, and steps with and without sums give the same state, bit for bit."""
+    _, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=seed)
+    s = lbm.Solver(cfg, precision="fp64", diag_every=1).set_geometry(arr).step(21)
+    t = lbm.Solver(cfg, precision="fp64").set_geometry(arr).step(20)
+    assert t.diagnostics() == s.diagnostics(compute=False)
+    s.close()
+    t.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("lattices", [1, 2, 4, 3, 5, 6, 7])
+def test_lattice_sets_and_the_readings_variant(env, lattices):
+    O, lbm = env
+    cfg, arr = W.random_state(45, 37, seed=3, lattices=lattices)
+    cfg = dict(cfg, readings=1, gx=3e-6, gy=-2e-6)
+    ref = O.from_workload((cfg, arr)).step(25).fields()
+    s = lbm.Solver(cfg, precision="fp64").set_geometry(arr).step(25)
+    _close(s.fields(), ref)
+    s.close()
+
+
+@pytest.mark.gpu
+def test_batch_of_columns_and_wide_grids_equals_single_grids(env):
+    """Each grid of a batch takes the kernel lbm_step takes: bit for bit."""
+    _, lbm = env
+    wls = [W.stefan(130, 5), W.random_state(40, 33, seed=1), W.random_state(50, 31, seed=2),
+           W.random_state(33, 64, seed=3)]
+    ss = [lbm.Solver(c, precision="fp64", diag_every=3).set_geometry(a) for c, a in wls]
+    b = lbm.Batch(ss).step(7).step(33)
+    for (cfg, arr), s in zip(wls, ss):
+        alone = lbm.Solver(cfg, precision="fp64", diag_every=3).set_geometry(arr).step(40)
+        fa, fb = alone.fields(), s.fields()
+        for k in FIELDS:
+            assert np.array_equal(fa[k], fb[k]), k
+        assert alone.diagnostics(compute=False) == s.diagnostics(compute=False)
+        alone.close()
+    b.close()
+
+
+@pytest.mark.gpu
+def test_a_nan_reaches_the_sums(env):
+    """One planted NaN is counted once by the step that reads it, and spreads."""
+    _, lbm = env
+    cfg, arr = W.random_state(40, 40, seed=2)
+    arr = {k: v.copy() for k, v in arr.items()}
+    arr["mask"][20, 20] = 0
+    arr["T"][20, 20] = np.nan
+    s = lbm.Solver(cfg, precision="fp64", diag_every=1).set_geometry(arr).step(1)
+    assert s.diagnostics(compute=False)["nonfinite"] == 1
+    assert s.step(1).diagnostics(compute=False)["nonfinite"] >= 5
+    s.close()
+
+
+def _fma(a, b, c):
+    return float(Fraction(a) * Fraction(b) + Fraction(c))  # one rounding, as the device's fma
+
+
+def test_third_order_reciprocal_is_within_an_ulp():
+    """r = r0 + r0 (e + e^2), e = 1 - b r0, from any seed within 2^-19 of 1 / b
+    (the hardware's approximation is nearer): less than one ulp off; and the
+    quotient corrected by its residual likewise."""
+    r = np.random.default_rng(5)
+    for _ in range(2000):
+        b = float(2.0 ** r.uniform(-30, 30))
+        r0 = float(Fraction(1) / Fraction(b) * (1 + Fraction(float(r.uniform(-1, 1)) * 2.0 ** -19)))
+        e = _fma(-b, r0, 1.0)
+        x = _fma(r0, _fma(e, e, e), r0)
+        exact = Fraction(1) / Fraction(b)
+        assert abs(Fraction(x) - exact) < Fraction(float(np.spacing(float(exact))))
+        a = float(r.uniform(-3, 3))
+        q0 = a * x
+        q = _fma(_fma(-q0, b, a), x, q0)
+        exact = Fraction(a) / Fraction(b)
+        assert abs(Fraction(q) - exact) < Fraction(float(np.spacing(abs(float(exact)))))
