@@ -280,14 +280,15 @@ void lbm_destroy(lbm_ctx* ctx);
  * of those grids, each tile evaluated by the same code as in lbm_step (the
  * results agree to the last bit where the compiler contracts both kernels'
  * copies of the arithmetic alike, as the FP64 build does, and otherwise to a
- * few roundings of the working precision).  This is how
+ * few roundings of the working precision).  LBM_FP64 batches take two launches
+ * per step and per 64 grids, and one more per 64 grids of few rows.  This is how
  * many small problems fill the GPU.  LBM_FP32 batches run as the batched
  * TMA-staged tile kernel (each tile's inputs copied to shared memory by the
  * tensor copies of its own context, one CTA per 32 x 8 tile; a copy that
  * does not arrive within the bounded wait makes that context's next read
- * return LBM_ERR_TIMEOUT), LBM_FP64 batches, and LBM_FP32 batches under the
- * environment variable LBM_BATCH_KERNEL=fused, as the one-CTA-per-tile
- * kernel loading from global memory.  The batch holds the context pointers
+ * return LBM_ERR_TIMEOUT), LBM_FP64 batches as lbm_step takes each grid, and
+ * LBM_FP32 batches under the environment variable LBM_BATCH_KERNEL=fused, as
+ * the one-CTA-per-tile kernel loading from global memory.  The batch holds the context pointers
  * only and allocates no device memory; the contexts stay usable on their own
  * (lbm_step, lbm_read_fields, diagnostics, checkpoints) and must outlive the
  * batch.
@@ -419,7 +420,11 @@ int lbm_adjoint_freezing(lbm_ctx* ctx, int64_t nsteps, int every, int observable
  * temperature; zero without a mask).  dT0 (host memory for
  * [ny][nx] doubles, or NULL): the gradient with respect to the initial
  * temperature field of lbm_set_geometry, node by node (the call must then
- * start at step 0, else LBM_ERR_STATE).  Other errors as
+ * start at step 0, else LBM_ERR_STATE).  Where all nsteps states (39 planes
+ * each) fit in an eighth of the device's free memory they are kept instead of
+ * the checkpoints and no segment is computed twice (LBM_ADJOINT_KEEP=0 in the
+ * environment: never); the results are the same.  Up to 1 GiB of work planes
+ * stays with the context until lbm_destroy.  Other errors as
  * lbm_adjoint_freezing. */
 int lbm_adjoint_coupled(lbm_ctx* ctx, int64_t nsteps, int every, int observable, int axis,
                         int index, double* value, double* grad, double* dT0, void* stream);
@@ -429,14 +434,16 @@ int lbm_adjoint_coupled(lbm_ctx* ctx, int64_t nsteps, int every, int observable,
  * and state and keeps the fastest for later lbm_step calls.  Variant v is
  * kernel form v / 2 with captured periods of at least 32 steps (v even) or
  * 256 (v odd).  Kernel forms (form ids; a context times those it has):
- * 0 one CTA per 32 x 8 tile loading from global memory (every precision);
- * 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one shared-memory
- * stage and one CTA per tile, LBM_FP64: the two-kernel split; 2 (float) the
+ * 0 float: one CTA per 32 x 8 tile loading from global memory, LBM_FP64 and
+ * tangents: the default, two node kernels of one thread per node (LBM_FP64
+ * grids of fewer than 32 rows and at most 32768 nodes: one CTA per 32 x 1
+ * tile); 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one
+ * shared-memory stage and one CTA per tile, LBM_FP64: the node kernels; 2 (float) the
  * TMA-staged kernel with two stages and two persistent CTAs per
  * multiprocessor (the copies of the next tile overlap the current one);
  * 3 (float) one stage and three persistent CTAs per multiprocessor; 4 one
- * CTA per 32 x 4 tile; 5 one CTA per 32 x 16 tile (4 and 5: LBM_FP32,
- * LBM_FP16S, LBM_FP64).  Tangent
+ * CTA per 32 x 4 tile; 5 one CTA per 32 x 16 tile, LBM_FP64: per 32 x 2 tile
+ * (4 and 5: LBM_FP32, LBM_FP16S, LBM_FP64).  Tangent
  * contexts 0.  Each variant runs steps_per_trial steps twice from the same
  * saved state (the first run warms up and captures; the second is timed
  * with CUDA events on `stream`).  The fastest variant is kept, unless the

@@ -24,7 +24,7 @@ cudaError_t launch_adjoint_init(const AdjArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_adjoint_reduce(const double* acc, const Geom& g, double* out, cudaStream_t s) {
-  lbm_adjoint_reduce_kernel<<<1, NT, 0, s>>>(acc, g, out);
+  lbm_adjoint_reduce_kernel<<<ADJ_NACC, RED_NT, 0, s>>>(acc, g, out);
   return cudaGetLastError();
 }
 
@@ -76,36 +76,6 @@ cudaError_t launch_frz_seed_crossing(const FrzArgs& a, double* phib, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_full_fields(const FullArgs& a, cudaStream_t s) {
-  lbm_full_fields_kernel<<<grid_dims(a.g), block_dims(), 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_full_k1(const FullArgs& a, cudaStream_t s) {
-  lbm_full_k1_kernel<<<grid_dims(a.g), block_dims(), 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_full_k2(const FullArgs& a, cudaStream_t s) {
-  lbm_full_k2_kernel<<<grid_dims(a.g), block_dims(), 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_full_seed_ff(const FullArgs& a, double* llag, cudaStream_t s) {
-  lbm_full_seed_ff_kernel<<<grid_dims(a.g), block_dims(), 0, s>>>(a, llag);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_full_seed_crossing(const FullArgs& a, double* phib, cudaStream_t s) {
-  lbm_full_seed_crossing_kernel<<<1, 32, 0, s>>>(a, phib);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_full_dT0(const FullArgs& a, const double* lam, double* out, cudaStream_t s) {
-  lbm_full_dT0_kernel<<<grid_dims(a.g), block_dims(), 0, s>>>(a, lam, out);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_adjoint_init_fields(const Geom& g, const double* gpop, const double* lag,
                                        const double* phi0, double* phi, double* fs,
                                        cudaStream_t s) {
@@ -114,3 +84,30 @@ cudaError_t launch_adjoint_init_fields(const Geom& g, const double* gpop, const 
 }
 
 }  // namespace lbmk
+
+namespace lbmn {
+
+static int rev_blocks(const RevArgs& a) { return (a.f.g.nodes + REV_NT - 1) / REV_NT; }
+
+cudaError_t launch_rev_step(const RevArgs& a, cudaStream_t s) {
+  rev_collide_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a);
+  rev_local_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rev_seed_ff(const RevArgs& a, double* llag, cudaStream_t s) {
+  rev_seed_ff_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a, llag);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rev_seed_crossing(const RevArgs& a, double* phib, cudaStream_t s) {
+  rev_seed_crossing_kernel<<<1, 32, 0, s>>>(a, phib);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rev_dT0(const RevArgs& a, const double* lam, double* out, cudaStream_t s) {
+  rev_dT0_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a, lam, out);
+  return cudaGetLastError();
+}
+
+}  // namespace lbmn

@@ -26,6 +26,7 @@ namespace lbmk {
 
 // accumulator planes: d/dT_wall[0..3], d/dlatent
 constexpr int ADJ_NACC = 5;
+constexpr int RED_NT = 1024;  // threads of their sums
 
 struct AdjArgs {
   Geom g;
@@ -285,31 +286,22 @@ static __global__ void __launch_bounds__(NT) lbm_adjoint_init_kernel(const AdjAr
 
 // Fixed-order sum of the accumulator planes over the grid (one CTA).
 #ifdef LBM_ADJOINT_KERNELS
-static __global__ void __launch_bounds__(NT) lbm_adjoint_reduce_kernel(const double* __restrict__ acc,
-                                                                Geom g, double* __restrict__ out) {
-  __shared__ double s[ADJ_NACC][NT / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int P = (int)g.plane;
-  double v[ADJ_NACC];
+static __global__ void __launch_bounds__(RED_NT) lbm_adjoint_reduce_kernel(
+    const double* __restrict__ acc, Geom g, double* __restrict__ out) {
+  __shared__ double s[RED_NT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = blockIdx.x;
+  const double* plane = acc + (long long)k * g.plane;
+  double v = 0.0;
+  for (int y = warp; y < g.ny; y += RED_NT / 32)
+    for (int x = lane; x < g.nx; x += 32) v += plane[(long long)y * g.pitch + x];
 #pragma unroll
-  for (int k = 0; k < ADJ_NACC; k++) v[k] = 0.0;
-  for (int y = 0; y < g.ny; y++)
-    for (int x = tid; x < g.nx; x += NT) {
-#pragma unroll
-      for (int k = 0; k < ADJ_NACC; k++) v[k] += acc[k * P + y * g.pitch + x];
-    }
-#pragma unroll
-  for (int k = 0; k < ADJ_NACC; k++) {
-    double w = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if (lane == 0) s[k][warp] = w;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s[warp] = v;
   __syncthreads();
-  if (tid < ADJ_NACC) {
+  if (tid == 0) {
     double t = 0.0;
-    for (int w = 0; w < NT / 32; w++) t += s[tid][w];
-    out[tid] = t;
+    for (int w = 0; w < RED_NT / 32; w++) t += s[w];
+    out[k] = t;
   }
 }
 #endif  // LBM_ADJOINT_KERNELS

@@ -89,11 +89,15 @@ struct lbm_ctx {
   uint64_t graph_gen;
   int graph_min;         // shortest captured period (32; lbm_autotune may change it)
   int graph_len;         // steps in the captured graph
+  // planes of lbm_adjoint_coupled, kept between calls up to kKeptWork bytes
+  double* work;
+  size_t work_len;       // doubles
   char err[512];
 };
 
 namespace {
 
+constexpr size_t kKeptWork = (size_t)1 << 30;
 const uint32_t kMagic = 0x4c424d46u;  // "LBMF"
 constexpr int kForms = 6;              // kernel form ids (form_available)
 constexpr int kAutotuneVariants = 2 * kForms;  // kernel forms x 2 captured periods
@@ -354,6 +358,28 @@ cudaError_t launch(lbm_ctx* c, int mode, bool diag, double* const* outs, cudaStr
   return lbmk::launch_step_f16s(a, mode, diag, s, ty);
 }
 
+// One FP64 step from the state at pops / lags into pops1 / lags1 by the
+// context's own kernel, with the node step's planes in `planes`.
+cudaError_t step_between(lbm_ctx* c, double* pops, double* lags, double* pops1, double* lags1,
+                         double* planes, cudaStream_t s) {
+  void* const keep[5] = {c->pop[0], c->pop[1], c->lag[0], c->lag[1], c->scratch};
+  const int cur = c->cur;
+  c->cur = 0;
+  c->pop[0] = pops;
+  c->pop[1] = pops1;
+  c->lag[0] = lags;
+  c->lag[1] = lags1;
+  c->scratch = planes;
+  const cudaError_t e = launch(c, lbmk::MODE_STEP, false, nullptr, s);
+  c->pop[0] = keep[0];
+  c->pop[1] = keep[1];
+  c->lag[0] = keep[2];
+  c->lag[1] = keep[3];
+  c->scratch = keep[4];
+  c->cur = cur;
+  return e;
+}
+
 // Steps of one captured period: the buffer parity repeats every two steps
 // and the diagnostic schedule every diag_every steps; short periods are
 // repeated up to at least 32 steps so that one graph launch covers many
@@ -452,7 +478,7 @@ void free_all(lbm_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   void* dev[] = {c->pop[0], c->pop[1], c->lag[0],     c->lag[1],    c->phi0,   c->mask,
                  c->diag_partial, c->diag_out, c->staging, c->in_stage,
-                 c->scratch, c->status, c->d_maps};
+                 c->scratch, c->status, c->d_maps, c->work};
   for (void* p : dev)
     if (p) cudaFree(p);
   if (c->h_diag) cudaFreeHost(c->h_diag);
@@ -1517,45 +1543,97 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
                 "readings == 0 and sigma > 0%s");
   cudaStream_t s = (cudaStream_t)stream;
   const size_t P = (size_t)c->g.plane;
-  const size_t pN = 27 * P, lN = lbmk::NLAG * P, stN = pN + lN;
-  const int64_t nck = (nsteps + every - 1) / every;
-  const int64_t seglen = std::min<int64_t>(every, nsteps);
-  // work planes: two adjoint sets of (27 populations, NLAG lags); phi, fs,
-  // rho; 7 stencil adjoints; the seed's phi adjoint and lag adjoints
-  const size_t setN = (27 + lbmk::NLAG) * P;
-  const size_t wN = 2 * setN + (3 + 7 + 1 + lbmk::NLAG) * P;
-  const int nacc = 10;
-  double *ck = nullptr, *seg = nullptr, *wk = nullptr, *acc = nullptr, *dout = nullptr,
-         *fin = nullptr;
-  cudaError_t e = cudaMalloc(&ck, nck * stN * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&seg, seglen * stN * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&wk, wN * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&acc, nacc * P * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&dout, 11 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&fin, stN * sizeof(double));
-  auto release = [&]() {
-    for (double* p : {ck, seg, wk, acc, dout, fin})
-      if (p) cudaFree(p);
+  const size_t pN = 27 * P, lN = lbmk::NLAG * P, stN = pN + lN;  // doubles per stored state
+  const int nacc = lbmn::FULL_NACC;
+  // one allocation: the kept states; then, cleared, two sets of adjoint
+  // populations and lags, the stencil and local adjoints, the crossing seed,
+  // the seed's lags and the accumulators; the states' fl and w, three field
+  // planes, the sums.  A slot is a state and the planes of its local pass,
+  // which the reverse takes from the forward step.
+  const size_t slotN = stN + lbmn::NSC * P;
+  const size_t clearN = 2 * stN + (lbmn::NSB + lbmn::NOWN + 1 + nacc) * P + lN;
+  const size_t rest = clearN + (2 + 3) * P + 16;
+  auto words = [&](int64_t ev) {
+    return (size_t)((nsteps + ev - 1) / ev - 1) * stN + (size_t)std::min<int64_t>(ev, nsteps) * slotN +
+           rest;
   };
-  if (e != cudaSuccess) {
-    release();
-    return cuda_fail(c, e, "adjoint allocation");
-  }
-  auto save = [&](double* dst) {
-    cudaError_t r = cudaMemcpyAsync(dst, c->pop[c->cur], pN * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    if (r == cudaSuccess)
-      r = cudaMemcpyAsync(dst + pN, c->lag[c->cur], lN * sizeof(double), cudaMemcpyDeviceToDevice, s);
+  // Where every state fits in an eighth of the free memory (LBM_ADJOINT_KEEP=0:
+  // never) all are kept and none is computed twice: 48 steps of the 256 x 256
+  // droplet take 0.9 GB and 7.9 ms against 10.3 ms with a checkpoint every 16
+  // steps.  The states, and so the results, are the same.
+  size_t freeb = 0, totalb = 0;
+  cudaError_t e = cudaMemGetInfo(&freeb, &totalb);
+  if (e != cudaSuccess) return cuda_fail(c, e, "adjoint");
+  const char* keep = std::getenv("LBM_ADJOINT_KEEP");
+  bool all = !(keep && std::strcmp(keep, "0") == 0) &&
+             (words(nsteps) <= c->work_len || words(nsteps) * sizeof(double) <= freeb / 8);
+  auto reserve = [&](size_t need) {
+    if (c->work_len >= need) return cudaSuccess;
+    if (c->work) cudaFree(c->work);
+    c->work = nullptr;
+    c->work_len = 0;
+    const cudaError_t r = cudaMalloc((void**)&c->work, need * sizeof(double));
+    if (r == cudaSuccess) c->work_len = need;
+    else cudaGetLastError();  // not the next launch's error
     return r;
   };
+  e = cudaSuccess;
+  if (all && reserve(words(nsteps)) != cudaSuccess) all = false;
+  if (!all) e = reserve(words(every));
+  if (e != cudaSuccess) return cuda_fail(c, e, "adjoint allocation");
+  if (all) every = (int)std::min<int64_t>(nsteps, 1 << 30);
+  const int64_t nck = (nsteps + every - 1) / every;
+  const int64_t seglen = std::min<int64_t>(every, nsteps);
+  // slot 0 serves each checkpoint in turn, the last one (the only one when
+  // all states are kept) from the start
+  double* seg = c->work;
+  double* ck = seg + seglen * slotN;
+  double* wk = ck + (nck - 1) * stN;
+  double* lb[2] = {wk, wk + stN};
+  double* sbp = wk + 2 * stN;
+  double* own = sbp + lbmn::NSB * P;
+  double* phib_seed = own + lbmn::NOWN * P;
+  double* seed_lag = phib_seed + P;
+  double* acc = seed_lag + lN;
+  double* flw = acc + nacc * P;
+  double* fld = flw + 2 * P;
+  double* dout = fld + 3 * P;
   int st = LBM_OK;
   const int64_t step0 = c->step;
-  std::vector<int> ckpar((size_t)nck);
-  for (int64_t k = 0; k < nsteps && e == cudaSuccess && st == LBM_OK; k++) {
-    if (k % every == 0) {
-      ckpar[(size_t)(k / every)] = c->cur;
-      e = save(ck + (k / every) * stN);
-    }
-    if (e == cudaSuccess) st = lbm_step(c, 1, s);
+  e = cudaMemsetAsync(wk, 0, clearN * sizeof(double), s);
+  auto slot = [&](int64_t j) { return seg + j * slotN; };
+  auto planes = [&](int64_t j) { return slot(j) + stN; };
+  auto copy_state = [&](double* dst, const double* pops, const double* lags) {
+    cudaError_t r = cudaMemcpyAsync(dst, pops, pN * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    if (r == cudaSuccess)
+      r = cudaMemcpyAsync(dst + pN, lags, lN * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    return r;
+  };
+  // states 1 ... len - 1 of a segment from its first, each step straight into
+  // its own slot
+  auto fill = [&](int64_t len) {
+    cudaError_t r = cudaSuccess;
+    for (int64_t j = 0; j + 1 < len && r == cudaSuccess; j++)
+      r = step_between(c, slot(j), slot(j) + pN, slot(j + 1), slot(j + 1) + pN, planes(j), s);
+    return r;
+  };
+  // forward: checkpoints, or every state
+  for (int64_t q = 0; q < nck && e == cudaSuccess && st == LBM_OK; q++) {
+    const int64_t len = std::min<int64_t>(every, nsteps - q * every);
+    e = copy_state(q == nck - 1 ? slot(0) : ck + q * stN, (const double*)c->pop[c->cur],
+                   (const double*)c->lag[c->cur]);
+    if (e == cudaSuccess && q < nck - 1) st = lbm_step(c, len, s);
+  }
+  // the last segment stays in its slots; its last step leads back into the context
+  if (e == cudaSuccess && st == LBM_OK) {
+    const int64_t len = nsteps - (nck - 1) * every;
+    e = fill(len);
+    if (e == cudaSuccess)
+      e = step_between(c, slot(len - 1), slot(len - 1) + pN, (double*)c->pop[c->cur ^ 1],
+                       (double*)c->lag[c->cur ^ 1], planes(len - 1), s);
+    c->cur ^= 1;
+    c->step += len;
+    c->last_stream = s;
   }
   double ffv = 0.0, inv_sum_w = 0.0;
   if (e == cudaSuccess && st == LBM_OK && observable == 0) {
@@ -1567,29 +1645,16 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
       inv_sum_w = 1.0 / d.material_volume;
     }
   }
-  const int parN = c->cur;
-  if (e == cudaSuccess && st == LBM_OK) e = save(fin);
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, nacc * P * sizeof(double), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(wk, 0, wN * sizeof(double), s);
   const double pi = 3.14159265358979323846;
-  double* lb[2] = {wk, wk + setN};
-  double* fld = wk + 2 * setN;
-  double* sbp = fld + 3 * P;
-  double* phib_seed = sbp + 7 * P;
-  double* seed_lag = phib_seed + P;
-  lbmk::FullArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.g = c->g;
-  a.c = c->cd;
-  a.phi0 = (const double*)c->phi0;
-  a.mask = (const unsigned char*)c->mask;
-  a.has_mask = c->g.has_mask;
-  a.phi = fld;
-  a.fs = fld + P;
-  a.rho = fld + 2 * P;
+  lbmn::RevArgs a;
+  std::memset((void*)&a, 0, sizeof(a));
+  a.f = node_args(c, c->nd);
+  a.f.lout = flw;
   a.sb = sbp;
+  a.own = own;
   a.acc = acc;
   a.dcos_dtheta = -std::sin(c->p.theta_deg * pi / 180.0) * (pi / 180.0);
+  a.inv_sigma = 1.0 / c->p.sigma;
   a.inv_sum_w = inv_sum_w;
   a.ff = ffv;
   a.axis = axis;
@@ -1601,58 +1666,64 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
     a.lam_out = lb[out];
     a.llag_out = lb[out] + pN;
   };
+  // The state at pops / lags becomes the one that is reversed.  With the
+  // local planes its own forward step left (and fl and w among the lags it
+  // wrote), or (null: the final state, and grids whose step is the fused
+  // tile, which leaves none) from a local pass of its own.
+  auto at_state = [&](const double* pops, const double* lags, double* local, double* next_lags) {
+    a.f.pin = pops;
+    a.f.lin = lags;
+    a.f.sc = local && c->node ? local : (double*)c->scratch;
+    a.f.lout = local && c->node ? next_lags : flw;
+    return local && c->node ? cudaSuccess : lbmn::launch_node_local(a.f, s);
+  };
   int cur_adj = 0;
   if (e == cudaSuccess && st == LBM_OK) {
-    a.pop = (const double*)c->pop[parN];
-    a.lag = (const double*)c->lag[parN];
-    e = lbmk::launch_full_fields(a, s);
-    set_io(1, 0);
+    e = at_state((const double*)c->pop[c->cur], (const double*)c->lag[c->cur], nullptr, nullptr);
+    set_io(1, 0);  // set 1 is still clear: no adjoint beyond the final state but the seed's
     if (observable == 0) {
-      if (e == cudaSuccess) e = lbmk::launch_full_seed_ff(a, seed_lag, s);
+      if (e == cudaSuccess) e = lbmn::launch_rev_seed_ff(a, seed_lag, s);
       a.llag_in = seed_lag;
     } else {
-      if (e == cudaSuccess) e = lbmk::launch_full_seed_crossing(a, phib_seed, s);
+      if (e == cudaSuccess) e = lbmn::launch_rev_seed_crossing(a, phib_seed, s);
       a.phib_seed = phib_seed;
     }
-    if (e == cudaSuccess) e = lbmk::launch_full_k2(a, s);
+    if (e == cudaSuccess) e = lbmn::launch_rev_step(a, s);
     a.phib_seed = nullptr;
   }
-  for (int64_t sg = nck - 1; sg >= 0 && e == cudaSuccess && st == LBM_OK; sg--) {
-    const int64_t k0 = sg * every, k1 = std::min<int64_t>(k0 + every, nsteps);
-    const int par = ckpar[(size_t)sg];
-    e = cudaMemcpyAsync(c->pop[par], ck + sg * stN, pN * sizeof(double), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(c->lag[par], ck + sg * stN + pN, lN * sizeof(double),
-                          cudaMemcpyDeviceToDevice, s);
-    c->cur = par;
-    c->step = step0 + k0;
-    c->gen++;
-    for (int64_t j = 0; j < k1 - k0 && e == cudaSuccess && st == LBM_OK; j++) {
-      e = save(seg + j * stN);
-      if (e == cudaSuccess) st = lbm_step(c, 1, s);
+  // reverse sweep: the states of each segment but the last again from its
+  // checkpoint, then back through them
+  for (int64_t q = nck - 1; q >= 0 && e == cudaSuccess && st == LBM_OK; q--) {
+    const int64_t len = std::min<int64_t>(every, nsteps - q * every);
+    if (q < nck - 1) {
+      e = copy_state(slot(0), ck + q * stN, ck + q * stN + pN);
+      if (e == cudaSuccess) e = fill(len);
     }
-    for (int64_t j = k1 - k0 - 1; j >= 0 && e == cudaSuccess && st == LBM_OK; j--) {
-      a.pop = seg + j * stN;
-      a.lag = seg + j * stN + pN;
+    for (int64_t j = len - 1; j >= 0 && e == cudaSuccess; j--) {
+      // the last state of a segment: the lags its step wrote are in the
+      // context (last segment) or were not computed again
+      const bool last = j == len - 1, have = !last || q == nck - 1;
+      e = at_state(slot(j), slot(j) + pN, have ? planes(j) : nullptr,
+                   last ? (double*)c->lag[c->cur] : slot(j + 1) + pN);
       set_io(cur_adj, cur_adj ^ 1);
-      e = lbmk::launch_full_fields(a, s);
-      if (e == cudaSuccess) e = lbmk::launch_full_k1(a, s);
-      if (e == cudaSuccess) e = lbmk::launch_full_k2(a, s);
+      if (e == cudaSuccess) e = lbmn::launch_rev_step(a, s);
       cur_adj ^= 1;
     }
   }
+  // a run from set_geometry's state: that state's dependence on L, theta and
+  // sigma (slot 0 holds it, and the planes are those of the last pass)
   if (e == cudaSuccess && st == LBM_OK && step0 == 0) {
     lbmk::AdjArgs ha;
     std::memset(&ha, 0, sizeof(ha));
     ha.g = c->g;
     ha.c = c->cd;
     ha.lam_in = lb[cur_adj] + 18 * P;
-    ha.lag = ck + pN;
+    ha.lag = slot(0) + pN;
     ha.acc = acc;
     e = lbmk::launch_adjoint_init(ha, s);
     if (e == cudaSuccess)
-      e = lbmk::launch_adjoint_init_fields(c->g, ck + 9 * P, ck + pN, (const double*)c->phi0, fld,
-                                           fld + P, s);
+      e = lbmk::launch_adjoint_init_fields(c->g, slot(0) + 9 * P, slot(0) + pN,
+                                           (const double*)c->phi0, fld, fld + P, s);
     lbmk::PhaseAdjArgs pa;
     std::memset(&pa, 0, sizeof(pa));
     pa.g = c->g;
@@ -1665,11 +1736,7 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
     pa.dcos_dtheta = a.dcos_dtheta;
     if (e == cudaSuccess) e = lbmk::launch_phase_adjoint_init(pa, s);
     if (e == cudaSuccess && dT0) {
-      // the checkpoint-0 state (initial populations and lags) in the
-      // reverse sweep's last recomputed slot; the field planes are reused
-      a.pop = ck;
-      a.lag = ck + pN;
-      e = lbmk::launch_full_dT0(a, lb[cur_adj] + 18 * P, fld, s);
+      e = lbmn::launch_rev_dT0(a, lb[cur_adj] + 18 * P, fld, s);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(dT0, fld, (size_t)c->p.nx * c->p.ny * sizeof(double),
                             cudaMemcpyDeviceToHost, s);
@@ -1680,20 +1747,18 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   if (e == cudaSuccess && st == LBM_OK) e = lbmk::launch_adjoint_reduce(acc + 5 * P, c->g, dout + 5, s);
   if (e == cudaSuccess && st == LBM_OK)
     e = cudaMemcpyAsync(hg, dout, sizeof(hg), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && st == LBM_OK)
-    e = cudaMemcpyAsync(c->pop[parN], fin, pN * sizeof(double), cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess && st == LBM_OK)
-    e = cudaMemcpyAsync(c->lag[parN], fin + pN, lN * sizeof(double), cudaMemcpyDeviceToDevice, s);
-  c->cur = parN;
-  c->step = step0 + nsteps;
-  c->gen++;
+  // the context's own buffers still hold the final state
   if (e == cudaSuccess && st == LBM_OK) st = lbm_compute_diagnostics(c, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  release();
+  if (c->work_len * sizeof(double) > kKeptWork) {  // not kept between calls
+    cudaFree(c->work);
+    c->work = nullptr;
+    c->work_len = 0;
+  }
   if (e != cudaSuccess) return cuda_fail(c, e, "adjoint");
   if (st != LBM_OK) return st;
   *value_out = observable == 0 ? ffv : hg[10];
-  for (int k = 0; k < lbmk::FULL_NACC; k++) grad[k] = hg[k];
+  for (int k = 0; k < lbmn::FULL_NACC; k++) grad[k] = hg[k];
   c->last_stream = s;
   return LBM_OK;
 }

@@ -83,6 +83,8 @@ namespace lbmn {
 template <typename R>
 cudaError_t launch_node(const NodeArgs<R, 2>& a, const ReadOut* ro, bool diag,
                         cudaStream_t s);
+// Its first kernel alone (the planes of a state).
+cudaError_t launch_node_local(const NodeArgs<double, 2>& a, cudaStream_t s);
 // Up to NODE_BATCH_GRIDS double grids in one pair of launches.
 cudaError_t launch_node_batch(const NodeBatch& b, bool diag, bool all, cudaStream_t s);
 

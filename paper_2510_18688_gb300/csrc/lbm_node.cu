@@ -64,6 +64,13 @@ cudaError_t launch_node(const NodeArgs<R, 2>& a, const ReadOut* ro, bool diag,
 template cudaError_t launch_node<double>(const NodeArgs<double, 2>&, const ReadOut*, bool, cudaStream_t);
 template cudaError_t launch_node<Dual>(const NodeArgs<Dual, 2>&, const ReadOut*, bool, cudaStream_t);
 
+cudaError_t launch_node_local(const NodeArgs<double, 2>& a, cudaStream_t s) {
+  const int wpb = warps_per_block(a.nwarps), nt = 32 * wpb, nb = (a.nwarps + wpb - 1) / wpb;
+  if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT)) node_local_kernel<double, 7><<<nb, nt, 0, s>>>(a);
+  else node_local_kernel<double, 0><<<nb, nt, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 // Batches: block t takes block t of the concatenated block lists of the
 // grids (its grid by bisection); a node's arithmetic and its warp's partial
 // sums are those of the single-grid kernels.

@@ -4,14 +4,13 @@
 //
 //   node_local    per node: the sums of the phase and enthalpy populations,
 //                 the inversion of Eq. (8), mdot, phi, w, fs and rho (rows
-//                 a1-a2); writes the four planes the neighbours' stencils
+//                 a1-a2); writes the three planes the neighbours' stencils
 //                 read -- phi, chi = phi + cos(theta) phi0 + cos(psi) fs (the
-//                 one Laplacian of Eq. (6) is that of chi), rho, and
-//                 pi = p_lag - rho / 3 (the modified force takes its
-//                 gradient) --, T, rho H and mdot for the node itself, and
-//                 fl and w straight into the next step's lag planes.
-//   node_collide  per node: the stencils from those planes through L1/L2,
-//                 mu_phi, forces, velocity and pressure, the three
+//                 one Laplacian of Eq. (6) is that of chi) and rho --, T, rho H
+//                 and mdot for the node itself, and fl and w straight into
+//                 the next step's lag planes.
+//   node_collide  per node: the stencils from those planes and the lagged
+//                 pressure through L1/L2, mu_phi, forces, velocity and pressure, the three
 //                 collisions, push streaming with the wall rules, lag store;
 //                 or (MODE_READ) the field read-out; diagnostics by warp.
 //
@@ -23,8 +22,8 @@
 // are linear over the grid, so a warp runs over row ends, and a grid of a
 // few thousand nodes is spread over all SMs by one-warp blocks; (c) the
 // collisions are written for the fewest operations: with the magic relation
-// 1/tau_s + 1/tau_a = 2 of the TRT, h_i* = (1/tau_a - 1) h_opp(i) + E_s + E_a,
-// so every population of every lattice costs one FMA and one add; the odd
+// 1/tau_s + 1/tau_a = 2 of the TRT, h_i* = q_i + (1/tau_a - 1) (h_o - q_o),
+// so a population of any lattice costs two or three operations; the odd
 // and quadratic equilibrium terms are dot products with vectors scaled once
 // per node (the diagonal weights are 1/4 or 1/2 of the axis ones, exact);
 // reciprocals take a hardware seed and one third-order iteration; clamps
@@ -100,7 +99,7 @@ template <int D>
 struct Lag {
   static constexpr int FL = 0, W = 1, P = 2, PHU = 3, Q = 3 + D, N = 4 + D;
 };
-enum { SC_PHI = 0, SC_CHI, SC_RHO, SC_PI, SC_T, SC_RHOH, SC_MDOT, NSC };
+enum { SC_PHI = 0, SC_CHI, SC_RHO, SC_T, SC_RHOH, SC_MDOT, NSC };
 
 // ---------------------------------------------------------------------------
 // arithmetic: R is float, double or Dual, K<R> its plain type (constants
@@ -370,27 +369,18 @@ struct Mix {
 // kernel 1
 // ---------------------------------------------------------------------------
 
-// population sums: one running sum in plane order in float, a tree (a short
-// dependent chain on the slow pipe) otherwise
-template <int D, typename R>
+// Population sums in the fixed orders of the fused step (2-D) and in plane
+// order (3-D): the initial state's sums decide by their last bits which side
+// of a clamp phi = -(1 - phi0) falls on in the gas beside a solid.
+template <int D, bool HEAT, typename R>
 __device__ __forceinline__ R sum_pops(const R* v) {
-  constexpr int Q = Lat<D>::Q;
-  if constexpr (std::is_same<R, float>::value) {
+  if constexpr (D == 2) {
+    return HEAT ? lbmk::sum_h(v) : lbmk::sum_g(v);
+  } else {
     R s = v[0];
 #pragma unroll
-    for (int i = 1; i < Q; i++) s += v[i];
+    for (int i = 1; i < Lat<D>::Q; i++) s += v[i];
     return s;
-  } else {
-    R t[(Q + 1) / 2];
-#pragma unroll
-    for (int i = 0; i < Q / 2; i++) t[i] = v[2 * i + 1] + v[2 * i + 2];
-    t[Q / 2] = v[0];
-#pragma unroll
-    for (int m = (Q + 1) / 2; m > 1; m = (m + 1) / 2) {
-#pragma unroll
-      for (int i = 0; i < m / 2; i++) t[i] = t[i] + t[m - 1 - i];
-    }
-    return t[0];
   }
 }
 
@@ -477,13 +467,12 @@ __device__ __forceinline__ void node_local(const NodeArgs<R, D>& a, int id) {
   const int n = node_pos<D>(g, id).n;
   const K<R> phi0 = plain(a.phi0[n]);
   const R flp = a.lin[L_::FL * P + n], wp = a.lin[L_::W * P + n], Qp = a.lin[L_::Q * P + n];
-  const R pp = a.lin[L_::P * P + n];
   R sg = R(0), sh = R(0);
   if (lat & LAT_PHASE) {
     R v[Q];
 #pragma unroll
     for (int i = 0; i < Q; i++) v[i] = a.pin[(Q + i) * P + n];
-    sg = sum_pops<D>(v);
+    sg = sum_pops<D, false>(v);
   }
   if (lat & LAT_HEAT) {
     R v[Q];
@@ -493,14 +482,13 @@ __device__ __forceinline__ void node_local(const NodeArgs<R, D>& a, int id) {
 #pragma unroll
       for (int i = 0; i < Q; i++) v[i] = a.pin[(2 * Q + i) * P + n];
     }
-    sh = sum_pops<D>(v);
+    sh = sum_pops<D, true>(v);
   }
   const LocalState<R> L = local_of<R, D>(c, lat, sg, sh, flp, wp, Qp, phi0);
   R* sc = a.sc + n;
   sc[SC_PHI * P] = L.phi;
   sc[SC_CHI * P] = mad(L.fs, c.cos_ps, mad(c.cos_th, phi0, L.phi));
   sc[SC_RHO * P] = L.rho;
-  sc[SC_PI * P] = mad(L.rho, K<R>(-1.0 / 3.0), pp);
   sc[SC_T * P] = L.T;
   sc[SC_RHOH * P] = L.rhoH;
   sc[SC_MDOT * P] = L.mdot;
@@ -537,27 +525,41 @@ __device__ __forceinline__ void gradient(const R* __restrict__ v, const Nbr<D>& 
   }
 }
 
-// 6 sum_i w_i (v(x + c_i) - v(x)); float subtracts the centre first (exact
-// for close neighbours), double sums the neighbours, which costs half the
-// operations and errs by an ulp or two of v, as v itself does
+// 6 sum_i w_i (v(x + c_i) - v(x)).  Float subtracts the centre from every
+// neighbour (exact for close ones); double from sums of 2, 4 and 8 neighbours,
+// half the operations.  Both are exactly zero for a uniform v -- sums of a
+// power of two of equal values do not round -- so a state at rest stays so
+// and phi stays exactly 0 inside a solid, where its sign decides clamps.
 template <typename R, int D>
 __device__ __forceinline__ R laplacian(const R* __restrict__ v, const R& vc, const Nbr<D>& b) {
   using L_ = Lat<D>;
-  R sa = R(0), sd = R(0);
+  R s[L_::NP];
 #pragma unroll
   for (int k = 0; k < L_::NP; k++) {
     const int i = L_::first(k);
-    R s;
     if constexpr (std::is_same<R, float>::value)
-      s = (v[toward<D>(b, i)] - vc) + (v[toward<D>(b, L_::opp(i))] - vc);
+      s[k] = (v[toward<D>(b, i)] - vc) + (v[toward<D>(b, L_::opp(i))] - vc);
     else
-      s = v[toward<D>(b, i)] + v[toward<D>(b, L_::opp(i))];
-    if (is_axis<D>(k)) sa = k == 0 ? s : sa + s;
-    else sd = k == D ? s : sd + s;
+      s[k] = v[toward<D>(b, i)] + v[toward<D>(b, L_::opp(i))];
   }
-  const R both = mad(sd, K<R>(6.0 * L_::w1 * L_::kd), mul(sa, K<R>(6.0 * L_::w1)));
-  if constexpr (std::is_same<R, float>::value) return both;
-  else return mad(vc, K<R>(-6.0 * (1.0 - L_::w0)), both);
+  R sa, sd;
+  if constexpr (std::is_same<R, float>::value) {
+    sa = s[0];
+    sd = s[D];
+#pragma unroll
+    for (int k = 1; k < D; k++) sa += s[k];
+#pragma unroll
+    for (int k = D + 1; k < L_::NP; k++) sd += s[k];
+  } else {
+    sa = mad(vc, K<R>(-4), s[0] + s[1]);
+    if constexpr (D == 2) {
+      sd = mad(vc, K<R>(-4), s[2] + s[3]);
+    } else {
+      sa += mad(vc, K<R>(-2), s[2]);
+      sd = mad(vc, K<R>(-8), (s[3] + s[4]) + (s[5] + s[6])) + mad(vc, K<R>(-4), s[7] + s[8]);
+    }
+  }
+  return mad(sd, K<R>(6.0 * L_::w1 * L_::kd), mul(sa, K<R>(6.0 * L_::w1)));
 }
 
 // Store of one post-collision population of direction i; behind a wall it
@@ -691,9 +693,9 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
     if (lat & LAT_FLOW) {
 #pragma unroll
       for (int i = 0; i < Q; i++) f[i] = a.pin[i * P + n];
-      R gr[D], gpi[D];
+      R gr[D], gp[D];
       gradient<R, D>(sc + SC_RHO * P, nb, gr);
-      gradient<R, D>(sc + SC_PI * P, nb, gpi);
+      gradient<R, D>(a.lin + G_::P * P + n, nb, gp);
       R j[D], snz = R(0);
       {
         R d[NP];
@@ -726,7 +728,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
         Gf[k] = mad(-rf, us, F[k]);
         uu = k == 0 ? u[k] * u[k] : mad(u[k], u[k], uu);
         // modified force (reading R-FT), lagged pressure (reading R-FP)
-        Ft[k] = F[k] - gpi[k];
+        Ft[k] = mad(gr[k], k_t(1.0 / 3.0), F[k] - gp[k]);
         uFt = k == 0 ? u[k] * Ft[k] : mad(u[k], Ft[k], uFt);
       }
       S = rho * mdot;
@@ -778,7 +780,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
           R v[Q];
 #pragma unroll
           for (int i = 0; i < Q; i++) v[i] = a.pin[(Q + i) * P + n];
-          bad = bad || !finite_word(sum_pops<D>(v));
+          bad = bad || !finite_word(sum_pops<D, false>(v));
         }
         bad = bad || !finite_word(rhoH);
       }
@@ -862,7 +864,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
         R gq[Q];
 #pragma unroll
         for (int i = 0; i < Q; i++) gq[i] = a.pin[(Q + i) * P + n];
-        if (DIAG) bad = bad || !finite_word(sum_pops<D>(gq));
+        if (DIAG) bad = bad || !finite_word(sum_pops<D, false>(gq));
         const R src = mul(phi * mdot, c.gcoef);
         const R em = mul(mu, c.itg_eta);
         const R Zs = em + src;
@@ -876,8 +878,9 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
         }
         {
           // itg (phi + (w_0 - 1) eta mu) + w_0 gcoef phi mdot
-          const R r0 = mad(Zs, k_t(L_::w0), mad(phi, c.itg, -em));
-          push<false>(a, out + Q * P, P, n, nb, 0, mad(gq[0], c.omg, r0));
+          // (the small terms first: one rounding at the size of phi)
+          const R r0 = mad(gq[0], c.omg, mad(Zs, k_t(L_::w0), -em));
+          push<false>(a, out + Q * P, P, n, nb, 0, mad(phi, c.itg, r0));
         }
 #pragma unroll
         for (int k = 0; k < NP; k++) {
@@ -912,21 +915,21 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
           for (int i = 0; i < Q; i++) hq[i] = a.pin[(2 * Q + i) * P + n];
         }
         if (DIAG) bad = bad || !finite_word(rhoH);
-        const R ia = rcp(mad(mix(c.lam), c.inv_rr3, k_t(0.5)));
-        const R is = R(2) - ia, am = add(ia, k_t(-1));
+        // By the magic relation 1/tau_s = 2 - 1/tau_a the collision is
+        // h_i* = q_i + (1/tau_a - 1) (h_o - q_o), o the opposite of i, with
+        // q = h_eq + w C T mdot / 2 (the source's factor 1 - 1/(2 tau_a) is
+        // half of 1/tau_s): a population at q stays there exactly
+        const R am = add(rcp(mad(mix(c.lam), c.inv_rr3, k_t(0.5))), k_t(-1));
         const R CT = rho * mix(c.cp) * T;
         CTm = CT * mdot;
-        const R src = mad(ia, k_t(-0.5), k_t(1)) * CTm;
         const R rrT = mul(T, c.rr);
-        const R iCT = is * CT;
-        const R Kn = mad(mul(iCT, k_t(-1.5)), uu, mad(is, rrT, src));
+        const R Kn = mad(CTm, k_t(0.5), mad(mul(CT, k_t(-1.5)), uu, rrT));
         const R Ka = mul(Kn, k_t(L_::w1)), Kd = mul(Kn, k_t(L_::w1 * L_::kd));
-        const R ya = mul(iCT, k_t(4.5 * L_::w1)), yd = mul(ya, k_t(L_::kd));
-        const R za = mul(ia * CT, k_t(3.0 * L_::w1)), zd = mul(za, k_t(L_::kd));
+        const R ya = mul(CT, k_t(4.5 * L_::w1)), yd = mul(ya, k_t(L_::kd));
+        const R za = mul(CT, k_t(3.0 * L_::w1)), zd = mul(za, k_t(L_::kd));
         {
-          // h0 (1 - is) + is (rho H - rr T) + w_0 (is (rr T - 3/2 C T uu) + src)
-          const R r0 = mad(Kn, k_t(L_::w0), is * (rhoH - rrT));
-          push<true>(a, out + 2 * Q * P, P, n, nb, 0, mad(hq[0], am, r0));
+          const R q0 = mad(Kn, k_t(L_::w0), rhoH - rrT);
+          push<true>(a, out + 2 * Q * P, P, n, nb, 0, mad(hq[0] - q0, am, q0));
         }
 #pragma unroll
         for (int k = 0; k < NP; k++) {
@@ -941,8 +944,9 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
             Ps = mad(cu * cu, yd, Kd);
             Pa = zd * cu;
           }
-          push<true>(a, out + 2 * Q * P, P, n, nb, i, mad(hq[o], am, Ps) + Pa);
-          push<true>(a, out + 2 * Q * P, P, n, nb, o, mad(hq[i], am, Ps) - Pa);
+          const R qi = Ps + Pa, qo = Ps - Pa;
+          push<true>(a, out + 2 * Q * P, P, n, nb, i, mad(hq[o] - qo, am, qi));
+          push<true>(a, out + 2 * Q * P, P, n, nb, o, mad(hq[i] - qi, am, qo));
         }
       }
       if (DIAG && (lat & LAT_FLOW)) bad = bad || !finite_word(ftot);

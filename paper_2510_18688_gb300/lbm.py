@@ -294,10 +294,11 @@ def lbm_adjoint_coupled(ctx, nsteps: int, every: int, observable: int, axis: int
 
 
 # kernel form ids of lbm_autotune (variant v = form v // 2, period v % 2)
-FORMS = ("one CTA per 32x8 tile", "float: TMA-staged, one stage / fp64: two-kernel split",
+FORMS = ("float: one CTA per 32x8 tile / fp64: by the grid",
+         "float: TMA-staged, one stage / fp64: node kernels",
          "float: TMA-staged, two stages, 2 persistent CTAs per SM",
          "float: TMA-staged, one stage, 3 persistent CTAs per SM", "one CTA per 32x4 tile",
-         "one CTA per 32x16 tile")
+         "float: one CTA per 32x16 tile / fp64: per 32x2 tile")
 N_VARIANTS = 2 * len(FORMS)
 VARIANTS = tuple(f"{f}, periods >= {p}" for f in FORMS for p in (32, 256))
 

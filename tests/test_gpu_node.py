@@ -114,6 +114,32 @@ def test_a_nan_reaches_the_sums(env):
     s.close()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(40, 33), (70, 12)])
+@pytest.mark.parametrize("every", [1, 5, 12, 50])
+def test_coupled_adjoint_with_all_states_equals_checkpoints(env, nx, ny, every, monkeypatch):
+    """Keeping every state or recomputing segments from checkpoints (the last
+    one short, of one state, or the only one): the same value, gradient, field
+    gradient and final state, bit for bit; and a second call goes on from it."""
+    _, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=3)
+    a = lbm.Solver(cfg, precision="fp64").set_geometry(arr)
+    b = lbm.Solver(cfg, precision="fp64").set_geometry(arr)
+    va, ga, ta = a.adjoint_coupled(23, observable=0, every=every, initial_T=True)
+    monkeypatch.setenv("LBM_ADJOINT_KEEP", "0")
+    vb, gb, tb = b.adjoint_coupled(23, observable=0, every=every, initial_T=True)
+    assert va == vb and ga == gb and np.array_equal(ta, tb)
+    assert a.adjoint_coupled(9, observable=1, axis=1, index=nx // 2, every=every) == \
+        b.adjoint_coupled(9, observable=1, axis=1, index=nx // 2, every=4) or \
+        np.isnan(a.crossings(1, nx // 2)[0])
+    assert a.steps_done == b.steps_done == 32
+    fa, fb = a.fields(), b.fields()
+    for k in FIELDS:
+        assert np.array_equal(fa[k], fb[k]), k
+    a.close()
+    b.close()
+
+
 def _fma(a, b, c):
     return float(Fraction(a) * Fraction(b) + Fraction(c))  # one rounding, as the device's fma
 
