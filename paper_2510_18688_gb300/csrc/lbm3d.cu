@@ -10,22 +10,19 @@
 // parameter, Eq. (10), the local part of Eq. (6)) is shared with the 2-D
 // step through lbm_kernels.cuh.
 //
-// A step is two kernels over the whole grid:
-//   lbm3_local_kernel    per node: the sums of the phase and enthalpy
-//                        populations, the inversion, mdot, phi, w, fs and
-//                        rho, stored as eight planes (phi, fs, rho for the
-//                        neighbours' stencils; T, fl, mdot, rho H, w for the
-//                        node itself);
-//   lbm3_collide_kernel  per node: the 18-neighbour stencils of phi, phi0,
-//                        fs, rho and the lagged pressure (neighbour planes
-//                        are read through L1/L2; a 32 x 4 x 2 block keeps
-//                        its halo in L1), mu_phi, forces, velocity and
-//                        pressure, the three collisions one lattice at a
-//                        time, push streaming with the wall rules, lag store.
-// The 2-D step fuses both halves with a recomputed halo ring; in 3-D the
+// A step is the two node kernels of lbm_node.cuh over the whole grid: the
+// local state of every node, then stencils, collisions and streaming.  The
+// 2-D float step fuses both halves with a recomputed halo ring; in 3-D the
 // ring of a 256-node tile is 2.2 times the tile, so the split form moves
-// fewer bytes: the eight local planes (32 B per node in FP32) instead of the
+// fewer bytes: eight local planes (32 B per node in FP32) instead of the
 // ring's population sums.
+//
+// What bounds it: FP32 the HBM traffic of the two passes, 201 + 529 B a node
+// against 516 B of a single pass (256 x 128 x 30 nodes: 35 + 93 us, 83 % and
+// 82 % of the copy rate; the collisions written pair by pair with general
+// streaming code took 178 us, at 24 warps an SM bound by latency; these fit
+// 64 registers and 32 warps, at 24 they take 98 us).  Double:
+// the FP64 pipe (131 x 67 x 30 nodes: 47 + 244 us against 61 + 621 us).
 //
 // Layout: structure-of-arrays planes of pitch * ny * nz elements (pitch =
 // nx rounded up to 32, planes to 64 elements); node (x, y, z) at
@@ -51,8 +48,8 @@ using lbmk::BC_DIRICHLET;
 using lbmk::BC_PERIODIC;
 
 constexpr int Q = 19;
-// thread block (x fastest) and the resident blocks per SM the FP32 collide
-// kernel is compiled for
+// thread block (x fastest; 32 x 8 x 1 measures the same) and the resident
+// blocks per SM the FP32 collide kernel is compiled for
 #ifndef LBM3_BY
 #define LBM3_BY 4
 #endif
@@ -60,7 +57,7 @@ constexpr int Q = 19;
 #define LBM3_BZ 2
 #endif
 #ifndef LBM3_MINB_F32
-#define LBM3_MINB_F32 3
+#define LBM3_MINB_F32 4
 #endif
 constexpr int BX = 32, BY = LBM3_BY, BZ = LBM3_BZ, NT = BX * BY * BZ;
 enum { L_FL = 0, L_W, L_P, L_PHUX, L_PHUY, L_PHUZ, L_Q, NLAG };
@@ -126,49 +123,6 @@ __device__ __forceinline__ int node(const Geom3& g, int x, int y, int z) {
   return (z * g.ny + y) * g.pitch + x;
 }
 
-// Streaming target of direction i from (x, y, z), or -1 with `wall` set to
-// the face it leaves through (the first wall crossed in the order x, y, z).
-__device__ __forceinline__ int stream_target(const Geom3& g, int x, int y, int z, int i,
-                                             int& wall) {
-  const int p[3] = {x + cx(i), y + cy(i), z + cz(i)};
-  const int n[3] = {g.nx, g.ny, g.nz};
-  int t[3];
-  wall = -1;
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    t[a] = p[a];
-    if (wall >= 0) continue;
-    if (p[a] < 0) {
-      if (g.bc[2 * a] == BC_PERIODIC) t[a] = p[a] + n[a]; else wall = 2 * a;
-    } else if (p[a] >= n[a]) {
-      if (g.bc[2 * a + 1] == BC_PERIODIC) t[a] = p[a] - n[a]; else wall = 2 * a + 1;
-    }
-  }
-  return wall >= 0 ? -1 : node(g, t[0], t[1], t[2]);
-}
-
-// Store of one post-collision population of direction i from node n; for
-// the enthalpy lattice (HEAT) a link leaving through a Dirichlet wall
-// returns by anti-bounce-back, through an adiabatic wall by bounce-back.
-template <typename R, bool HEAT, typename I>
-__device__ __forceinline__ void push(const Args3<R>& a, R* __restrict__ plane0, I P, int i,
-                                     int x, int y, int z, int n, bool inner, R v) {
-  const Geom3& g = a.g;
-  if (inner) {
-    plane0[i * P + n + (cz(i) * g.ny + cy(i)) * g.pitch + cx(i)] = v;
-  } else {
-    int wall;
-    const int t = stream_target(g, x, y, z, i, wall);
-    if (t >= 0) {
-      plane0[i * P + t] = v;
-    } else {
-      if (HEAT && g.bc[wall] == BC_DIRICHLET) v = -v + R(2) * wq<R>(i) * a.c.rr * a.T_wall[wall];
-      plane0[opp(i) * P + n] = v;
-    }
-  }
-}
-
-
 // Enthalpy populations of a cold-mask node: the equilibrium of Eq. (25) at
 // T_cold with u = 0, at the node's weight w and phi0 (applied when the
 // populations are read).
@@ -195,317 +149,61 @@ __device__ __forceinline__ R sum19(const R* v) {
 }
 
 // ---------------------------------------------------------------------------
-// kernel 1: local state of every node
+// the step and the read-out: the node kernels of lbm_node.cuh.  Float takes
+// 32 x 4 x 2 blocks, whose stencil halos stay in L1; double and tangents,
+// which the FP64 pipe bounds, linear node ids (no idle lanes at row ends).
 // ---------------------------------------------------------------------------
 
-// I: the type of plane offsets (int while 57 population planes fit 31
-// bits, which keeps the index arithmetic in 32-bit registers; long long for
-// larger grids)
-template <typename R, typename I>
-__global__ void __launch_bounds__(NT) lbm3_local_kernel(const Args3<R> a) {
-  const Geom3& g = a.g;
-  const Coef<R>& c = a.c;
-  const int x = blockIdx.x * BX + threadIdx.x;
-  const int y = blockIdx.y * BY + threadIdx.y;
-  const int z = blockIdx.z * BZ + threadIdx.z;
-  if (x >= g.nx || y >= g.ny || z >= g.nz) return;
-  const I P = (I)g.plane;
-  const int n = node(g, x, y, z);
-  const int lat = g.lattices;
-  const R phi0 = a.phi0[n];
-  const R flp = a.lin[L_FL * P + n], wp = a.lin[L_W * P + n], Qp = a.lin[L_Q * P + n];
-  R sg = R(0), sh = R(0);
-  if (lat & LAT_PHASE) {
-    R v[Q];
-#pragma unroll
-    for (int i = 0; i < Q; i++) v[i] = a.pin[(Q + i) * P + n];
-    sg = sum19(v);
-  }
-  if (lat & LAT_HEAT) {
-    R v[Q];
-    if (g.has_mask && a.mask[n]) {
-      cold_mask_h19(c, wp, phi0, v);
-    } else {
-#pragma unroll
-      for (int i = 0; i < Q; i++) v[i] = a.pin[(2 * Q + i) * P + n];
-    }
-    sh = sum19(v);
-  }
-  const lbmk::Local<R> L = lbmk::local_state(c, lat, sg, sh, flp, wp, Qp, phi0);
-  R* loc = a.loc + n;
-  loc[S_PHI * P] = L.phi;
-  loc[S_FS * P] = L.fs;
-  loc[S_RHO * P] = L.rho;
-  loc[S_T * P] = L.T;
-  loc[S_FL * P] = L.fl;
-  loc[S_MDOT * P] = L.mdot;
-  loc[S_RHOH * P] = L.rhoH;
-  loc[S_W * P] = L.w;
-}
-
-// ---------------------------------------------------------------------------
-// kernel 2: stencils, macroscopic fields, collisions, streaming
-// ---------------------------------------------------------------------------
-
+constexpr int NLIN = 128;
 template <typename R>
-struct Macro3 {
-  R u[3], uu, pr, S, Ft[3], uFt, G[3], tauf, muphi, phu[3], cap;
-};
-
-// Flow collision Eqs. (11), (14)-(16) over the opposite pairs (i, i + 1):
-// the terms even in c_i are shared by the pair, the odd ones change sign.
-template <typename R, typename I>
-__device__ __forceinline__ void collide_flow(const Args3<R>& a, R* out, I P, int x, int y,
-                                             int z, int n, bool inner, const R* f, R rho,
-                                             const Macro3<R>& M) {
-  const R itau = lbmk::qdiv(R(1), M.tauf);
-  const R omi = R(1) - itau;
-  const R fcoef = R(1) - R(0.5) * itau;
-  const bool iso = (a.c.readings & 1u) != 0;
-  const R sym0 = rho * (-R(1.5) * M.uu);
-  const R fsym0 = M.S - R(3) * M.uFt;
-  {
-    R F0 = fsym0;
-    if (iso) F0 += M.S * (R(0) - R(1)) * R(1.5);
-    const R feq0 = M.pr * R(3) * (wq<R>(0) - R(1)) + rho * wq<R>(0) * (-R(1.5) * M.uu);
-    push<R, false, I>(a, out, P, 0, x, y, z, n, inner, f[0] * omi + itau * feq0 + fcoef * wq<R>(0) * F0);
-  }
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const int o = i + 1;
-    const R wi = wq<R>(i);
-    const R cu = R(cx(i)) * M.u[0] + R(cy(i)) * M.u[1] + R(cz(i)) * M.u[2];
-    const R cG = R(cx(i)) * M.G[0] + R(cy(i)) * M.G[1] + R(cz(i)) * M.G[2];
-    const R cFt = R(cx(i)) * M.Ft[0] + R(cy(i)) * M.Ft[1] + R(cz(i)) * M.Ft[2];
-    const R eqS = M.pr * R(3) + rho * (R(4.5) * cu * cu) + sym0;
-    const R eqA = rho * (R(3) * cu);
-    R srcS = fsym0 + R(9) * cu * cFt;
-    if (iso) srcS += M.S * (R(cx(i) * cx(i) + cy(i) * cy(i) + cz(i) * cz(i)) - R(1)) * R(1.5);
-    const R srcA = R(3) * cG;
-    const R Ps = wi * (itau * eqS + fcoef * srcS);
-    const R Pa = wi * (itau * eqA + fcoef * srcA);
-    push<R, false, I>(a, out, P, i, x, y, z, n, inner, f[i] * omi + Ps + Pa);
-    push<R, false, I>(a, out, P, o, x, y, z, n, inner, f[o] * omi + Ps - Pa);
-  }
+constexpr bool kTiled = std::is_same<R, float>::value;
+template <typename R>
+constexpr int kThreads = kTiled<R> ? NT : NLIN;
+template <typename R>
+constexpr int min_blocks() {
+  return kTiled<R> ? LBM3_MINB_F32 : (std::is_same<R, double>::value ? 4 : 2);
 }
 
-// Phase-field collision Eqs. (18)-(20).
+// The lattice set is read at run time: the branches keep the compiler from
+// hoisting all 57 population loads to the top (with the set fixed it spills
+// 376 B a thread at 80 registers).
 template <typename R, typename I>
-__device__ __forceinline__ void collide_phase(const Args3<R>& a, R* out, I P, int x, int y,
-                                              int z, int n, bool inner, const R* gq, R phi,
-                                              R mdot, const R* phup, const Macro3<R>& M) {
-  const Coef<R>& c = a.c;
-  const R itg = c.inv_tau_g;
-  const R omg = R(1) - itg;
-  const R gcoef = R(1) - R(0.5) * itg;
-  const R emu = c.eta * M.muphi;
-  const R Zs = itg * emu + gcoef * phi * mdot;
-  R V[3];
-#pragma unroll
-  for (int k = 0; k < 3; k++) V[k] = R(3) * (itg * M.phu[k] + gcoef * (M.phu[k] - phup[k]));
-  {
-    const R geq0 = phi + (wq<R>(0) - R(1)) * emu;
-    push<R, false, I>(a, out, P, 0, x, y, z, n, inner,
-                   gq[0] * omg + itg * geq0 + gcoef * wq<R>(0) * phi * mdot);
-  }
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const int o = i + 1;
-    const R wi = wq<R>(i);
-    const R Ps = wi * Zs;
-    const R Pa = wi * (R(cx(i)) * V[0] + R(cy(i)) * V[1] + R(cz(i)) * V[2]);
-    push<R, false, I>(a, out, P, i, x, y, z, n, inner, gq[i] * omg + Ps + Pa);
-    push<R, false, I>(a, out, P, o, x, y, z, n, inner, gq[o] * omg + Ps - Pa);
-  }
-}
-
-// Enthalpy TRT collision Eqs. (23)-(27) with the magic relation.
-template <typename R, typename I>
-__device__ __forceinline__ void collide_heat(const Args3<R>& a, R* out, I P, int x, int y,
-                                             int z, int n, bool inner, const R* h, R fs, R w,
-                                             R T, R rhoH, R mdot, const Macro3<R>& M) {
-  const Coef<R>& c = a.c;
-  const R lam = lbmk::interp(fs, w, c.lam_s, c.lam_l, c.lam_g);
-  const R taua = R(0.5) + lam * c.inv_rr3;
-  const R ia = lbmk::qdiv(R(1), taua), is = R(2) - ia;
-  const R hcoef = R(1) - R(0.5) * ia;
-  const R CT = M.cap * T;
-  const R Hsrc = hcoef * CT * mdot;
-  const R rrT = c.rr * T;
-  {
-    const R heq0 = rhoH - rrT + wq<R>(0) * (rrT - CT * M.uu * R(1.5));
-    push<R, true, I>(a, out, P, 0, x, y, z, n, inner, h[0] - (h[0] - heq0) * is + wq<R>(0) * Hsrc);
-  }
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const int o = i + 1;
-    const R wi = wq<R>(i);
-    const R cu = R(cx(i)) * M.u[0] + R(cy(i)) * M.u[1] + R(cz(i)) * M.u[2];
-    const R es = wi * (rrT + CT * (R(4.5) * cu * cu - R(1.5) * M.uu));
-    const R ea = wi * (CT * (R(3) * cu));
-    const R hs = R(0.5) * (h[i] + h[o]), ha = R(0.5) * (h[i] - h[o]);
-    const R Da = (ha - ea) * ia;
-    const R Ds = (hs - es) * is - wi * Hsrc;
-    push<R, true, I>(a, out, P, i, x, y, z, n, inner, h[i] - Da - Ds);
-    push<R, true, I>(a, out, P, o, x, y, z, n, inner, h[o] + Da - Ds);
+__global__ void __launch_bounds__(kThreads<R>)
+    lbm3_local_kernel(const __grid_constant__ lbmn::NodeArgs<R, 3> a) {
+  if constexpr (kTiled<R>) {
+    const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
+    const int z = blockIdx.z * BZ + threadIdx.z;
+    if (x < a.g.n[0] && y < a.g.n[1] && z < a.g.n[2])
+      lbmn::node_local<R, 3, 0, I>(a, lbmn::node_at(a.g, x, y, z).n);
+  } else {
+    lbmn::node_local_linear<R, 3, 0, I>(a, blockIdx.x * blockDim.x + threadIdx.x);
   }
 }
 
 template <typename R, bool READ, typename I>
-__global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? LBM3_MINB_F32 : (sizeof(R) == 8 ? 2 : 1)))
-    lbm3_collide_kernel(const Args3<R> a) {
-  const Geom3& g = a.g;
-  const Coef<R>& c = a.c;
-  const int x = blockIdx.x * BX + threadIdx.x;
-  const int y = blockIdx.y * BY + threadIdx.y;
-  const int z = blockIdx.z * BZ + threadIdx.z;
-  if (x >= g.nx || y >= g.ny || z >= g.nz) return;
-  const I P = (I)g.plane;
-  const int n = node(g, x, y, z);
-  const int lat = g.lattices;
-  const R* loc = a.loc;
-  const R phi = loc[S_PHI * P + n], fs = loc[S_FS * P + n], rho = loc[S_RHO * P + n];
-  const R T = loc[S_T * P + n], fl = loc[S_FL * P + n], mdot = loc[S_MDOT * P + n];
-  const R rhoH = loc[S_RHOH * P + n], w = loc[S_W * P + n];
-  const R phi0 = a.phi0[n];
+__device__ __forceinline__ void collide3(const lbmn::NodeArgs<R, 3>& a, const lbmn::ReadOut* ro) {
+  if constexpr (kTiled<R>) {
+    const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
+    const int z = blockIdx.z * BZ + threadIdx.z;
+    if (x < a.g.n[0] && y < a.g.n[1] && z < a.g.n[2])
+      lbmn::node_collide<R, 3, 0, READ, false, I>(a, ro, true, lbmn::node_at(a.g, x, y, z), 0);
+  } else {
+    lbmn::node_collide_linear<R, 3, 0, READ, false, I>(a, ro,
+                                                      blockIdx.x * blockDim.x + threadIdx.x);
+  }
+}
 
-  // isotropic stencils (reading R-FD) over the 18 neighbours; wall axes
-  // mirror the boundary node (zero normal gradient)
-  R gph[3] = {R(0), R(0), R(0)}, gr[3] = {R(0), R(0), R(0)}, gp[3] = {R(0), R(0), R(0)};
-  R lphi = R(0), lphi0 = R(0), lfs = R(0);
-#pragma unroll
-  for (int i = 1; i < Q; i++) {
-    const int xx = wrap_or_clamp(x + cx(i), g.nx, g.bc[0], g.bc[1]);
-    const int yy = wrap_or_clamp(y + cy(i), g.ny, g.bc[2], g.bc[3]);
-    const int zz = wrap_or_clamp(z + cz(i), g.nz, g.bc[4], g.bc[5]);
-    const int m = node(g, xx, yy, zz);
-    const R wi = wq<R>(i);
-    const R vphi = loc[S_PHI * P + m];
-    if (lat & LAT_PHASE) {
-      const R vphi0 = a.phi0[m], vfs = loc[S_FS * P + m];
-      gph[0] += wi * R(cx(i)) * vphi;
-      gph[1] += wi * R(cy(i)) * vphi;
-      gph[2] += wi * R(cz(i)) * vphi;
-      lphi += R(2) * wi * (vphi - phi);
-      lphi0 += R(2) * wi * (vphi0 - phi0);
-      lfs += R(2) * wi * (vfs - fs);
-    }
-    if (lat & LAT_FLOW) {
-      const R vrho = loc[S_RHO * P + m], vp = a.lin[L_P * P + m];
-      gr[0] += wi * R(cx(i)) * vrho;
-      gr[1] += wi * R(cy(i)) * vrho;
-      gr[2] += wi * R(cz(i)) * vrho;
-      gp[0] += wi * R(cx(i)) * vp;
-      gp[1] += wi * R(cy(i)) * vp;
-      gp[2] += wi * R(cz(i)) * vp;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    gph[k] *= R(3);
-    gr[k] *= R(3);
-    gp[k] *= R(3);
-  }
-  lphi *= R(3); lphi0 *= R(3); lfs *= R(3);
+template <typename R, typename I>
+__global__ void __launch_bounds__(kThreads<R>, min_blocks<R>())
+    lbm3_collide_kernel(const __grid_constant__ lbmn::NodeArgs<R, 3> a) {
+  collide3<R, false, I>(a, nullptr);
+}
 
-  Macro3<R> M;
-  M.muphi = R(0);
-  R F[3];
-  {
-    R Fs[3] = {R(0), R(0), R(0)};
-    if (lat & LAT_PHASE) {
-      M.muphi = lbmk::chem_local(c, phi, phi0, fs) -
-                c.klap * (lphi + c.cos_th * lphi0 + c.cos_ps * lfs);
-#pragma unroll
-      for (int k = 0; k < 3; k++) Fs[k] = M.muphi * gph[k];
-    }
-    F[0] = Fs[0] + rho * c.gx;
-    F[1] = Fs[1] + rho * c.gy;
-    F[2] = Fs[2] + rho * a.gz;
-  }
-  M.u[0] = M.u[1] = M.u[2] = R(0);
-  M.uu = R(0);
-  M.pr = R(0);
-  R f[Q];
-  if (lat & LAT_FLOW) {
-#pragma unroll
-    for (int i = 0; i < Q; i++) f[i] = a.pin[i * P + n];
-    R j[3] = {R(0), R(0), R(0)}, snz = R(0);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      j[0] += R(cx(i)) * f[i];
-      j[1] += R(cy(i)) * f[i];
-      j[2] += R(cz(i)) * f[i];
-      if (i > 0) snz += f[i];
-    }
-    const R mu = lbmk::interp(fs, w, c.mu_s, c.mu_l, c.mu_g);
-    const R irho = lbmk::qdiv(R(1), rho);
-    // Eq. (17a,b) with the penalty force f = fs (u_s - u*), u_s = 0
-    R fp[3];
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const R us = (j[k] + R(0.5) * F[k]) * irho;
-      fp[k] = -fs * us;
-      M.u[k] = us + R(0.5) * fp[k];
-    }
-    M.uu = M.u[0] * M.u[0] + M.u[1] * M.u[1] + M.u[2] * M.u[2];
-    M.S = rho * mdot + M.u[0] * gr[0] + M.u[1] * gr[1] + M.u[2] * gr[2];
-    // modified force (reading R-FT) with the lagged pressure (reading R-FP)
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      M.Ft[k] = F[k] - (gp[k] - gr[k] * R(1.0 / 3.0));
-      M.G[k] = F[k] + rho * fp[k];
-    }
-    M.uFt = M.u[0] * M.Ft[0] + M.u[1] * M.Ft[1] + M.u[2] * M.Ft[2];
-    M.tauf = R(3) * mu * irho + R(0.5);
-    // F_0 of Eq. (16) and Eq. (17c)
-    R F0 = wq<R>(0) * (M.S + (R(0) - R(2) / R(3) * M.uFt) * R(4.5));
-    if (c.readings & 1u) F0 += wq<R>(0) * (M.S * (R(0) - R(1)) * R(1.5));
-    const R s0 = wq<R>(0) * (-M.uu * R(1.5));
-    M.pr = (R(1) / R(3)) / (R(1) - wq<R>(0)) *
-           (snz + R(0.5) * M.S + (M.tauf - R(0.5)) * F0 + rho * s0);
-  }
-#pragma unroll
-  for (int k = 0; k < 3; k++) M.phu[k] = phi * M.u[k];
-  M.cap = rho * lbmk::interp(fs, w, c.cp_s, c.cp_l, c.cp_g);
-
-  if (READ) {
-    const long long N = (long long)g.nx * g.ny * g.nz;
-    const long long d = ((long long)z * g.ny + y) * g.nx + x;
-    const R vals[NFIELD3] = {phi, fs, fl, T, rhoH, M.pr, M.u[0], M.u[1], M.u[2],
-                             rho, M.muphi, w, mdot};
-#pragma unroll
-    for (int k = 0; k < NFIELD3; k++) lbmk::put_out(a.fld + k * N, d, NFIELD3 * N, vals[k]);
-    return;
-  }
-
-  const bool inner = x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1;
-  R* out = a.pout;
-  if (lat & LAT_FLOW) collide_flow(a, out, P, x, y, z, n, inner, f, rho, M);
-  if (lat & LAT_PHASE) {
-    R gq[Q];
-#pragma unroll
-    for (int i = 0; i < Q; i++) gq[i] = a.pin[(Q + i) * P + n];
-    const R phup[3] = {a.lin[L_PHUX * P + n], a.lin[L_PHUY * P + n], a.lin[L_PHUZ * P + n]};
-    collide_phase(a, out + Q * P, P, x, y, z, n, inner, gq, phi, mdot, phup, M);
-  }
-  if (lat & LAT_HEAT) {
-    R hq[Q];
-    if (g.has_mask && a.mask[n]) {
-      cold_mask_h19(c, a.lin[L_W * P + n], phi0, hq);
-    } else {
-#pragma unroll
-      for (int i = 0; i < Q; i++) hq[i] = a.pin[(2 * Q + i) * P + n];
-    }
-    collide_heat(a, out + 2 * Q * P, P, x, y, z, n, inner, hq, fs, w, T, rhoH, mdot, M);
-  }
-  a.lout[L_FL * P + n] = fl;
-  a.lout[L_W * P + n] = w;
-  a.lout[L_P * P + n] = (lat & LAT_FLOW) ? M.pr : R(0);
-  a.lout[L_PHUX * P + n] = (lat & LAT_PHASE) ? M.phu[0] : R(0);
-  a.lout[L_PHUY * P + n] = (lat & LAT_PHASE) ? M.phu[1] : R(0);
-  a.lout[L_PHUZ * P + n] = (lat & LAT_PHASE) ? M.phu[2] : R(0);
-  a.lout[L_Q * P + n] = (lat & LAT_HEAT) ? M.cap * T * mdot : R(0);
+template <typename R, typename I>
+__global__ void __launch_bounds__(kThreads<R>, min_blocks<R>())
+    lbm3_read_kernel(const __grid_constant__ lbmn::NodeArgs<R, 3> a,
+                     const __grid_constant__ lbmn::ReadOut ro) {
+  collide3<R, true, I>(a, &ro);
 }
 
 // ---------------------------------------------------------------------------
@@ -724,6 +422,9 @@ struct lbm3_ctx {
   lbmk::Coef<float> cf;
   lbmk::Coef<double> cd;
   lbmk::Coef<lbmk::Dual> ct;
+  lbmn::NodeCoef<float, 3> nf;  // the step's constants
+  lbmn::NodeCoef<double, 3> nd;
+  lbmn::NodeCoef<lbmk::Dual, 3> nt;
   double h_tan[lbm3::NDIAG3];  // derivative sums of the last diagnostics
   int64_t tan_step;
   void* pop[2];
@@ -787,26 +488,71 @@ lbm3::Args3<R> args3(lbm3_ctx* c, const lbmk::Coef<R>& coef) {
   return a;
 }
 
-// one step (read == false) or the read-out of the current state's fields
-// into c->fld (read == true)
 template <typename R>
-cudaError_t launch3(lbm3_ctx* c, const lbmk::Coef<R>& coef, bool read, cudaStream_t s) {
-  const lbm3::Args3<R> a = args3<R>(c, coef);
-  if (c->g.plane * 57 < (1LL << 31)) {
-    lbm3::lbm3_local_kernel<R, int><<<grid3(c->g), block3(), 0, s>>>(a);
-    if (read) lbm3::lbm3_collide_kernel<R, true, int><<<grid3(c->g), block3(), 0, s>>>(a);
-    else lbm3::lbm3_collide_kernel<R, false, int><<<grid3(c->g), block3(), 0, s>>>(a);
-  } else {
-    lbm3::lbm3_local_kernel<R, long long><<<grid3(c->g), block3(), 0, s>>>(a);
-    if (read) lbm3::lbm3_collide_kernel<R, true, long long><<<grid3(c->g), block3(), 0, s>>>(a);
-    else lbm3::lbm3_collide_kernel<R, false, long long><<<grid3(c->g), block3(), 0, s>>>(a);
+lbmn::NodeArgs<R, 3> node_args3(lbm3_ctx* c, const lbmn::NodeCoef<R, 3>& coef) {
+  lbmn::NodeArgs<R, 3> a;
+  std::memset((void*)&a, 0, sizeof(a));
+  const lbm3::Geom3& g = c->g;
+  const int n[3] = {g.nx, g.ny, g.nz};
+  for (int k = 0; k < 3; k++) a.g.n[k] = n[k];
+  a.g.pitch = g.pitch;
+  a.g.nodes = g.nx * g.ny * g.nz;
+  a.g.dx = lbmn::make_fastdiv((unsigned)g.nx);
+  a.g.dy = lbmn::make_fastdiv((unsigned)g.ny);
+  a.g.plane = g.plane;
+  for (int k = 0; k < 6; k++) a.g.bc[k] = g.bc[k];
+  a.g.lattices = g.lattices;
+  a.g.has_mask = g.has_mask;
+  a.c = coef;
+  a.pin = (const R*)c->pop[c->cur];
+  a.pout = (R*)c->pop[c->cur ^ 1];
+  a.lin = (const R*)c->lag[c->cur];
+  a.lout = (R*)c->lag[c->cur ^ 1];
+  a.phi0 = (const R*)c->phi0;
+  a.mask = c->mask;
+  a.sc = (R*)c->loc;
+  return a;
+}
+
+// The step (ro null) or the read-out of the current state's fields into the
+// planes of ro.  The read-out leaves the state alone (it writes fl and w into
+// the lag planes the next step will overwrite).
+template <typename R, typename I>
+void launch_step3(const lbmn::NodeArgs<R, 3>& a, const lbmn::ReadOut* ro, dim3 gd, dim3 bd,
+                  cudaStream_t s) {
+  lbm3::lbm3_local_kernel<R, I><<<gd, bd, 0, s>>>(a);
+  if (ro) lbm3::lbm3_read_kernel<R, I><<<gd, bd, 0, s>>>(a, *ro);
+  else lbm3::lbm3_collide_kernel<R, I><<<gd, bd, 0, s>>>(a);
+}
+
+template <typename R>
+cudaError_t launch3(lbm3_ctx* c, const lbmn::NodeCoef<R, 3>& coef, const lbmn::ReadOut* ro,
+                    cudaStream_t s) {
+  const lbmn::NodeArgs<R, 3> a = node_args3<R>(c, coef);
+  dim3 gd = grid3(c->g), bd = block3();
+  if (!lbm3::kTiled<R>) {
+    gd = dim3((unsigned)((a.g.nodes + lbm3::NLIN - 1) / lbm3::NLIN));
+    bd = dim3(lbm3::NLIN);
   }
+  // offsets are 32-bit while 57 planes allow
+  if (c->g.plane * 57 < (1LL << 31)) launch_step3<R, int>(a, ro, gd, bd, s);
+  else launch_step3<R, long long>(a, ro, gd, bd, s);
   return cudaGetLastError();
 }
 
-cudaError_t launch3(lbm3_ctx* c, bool read, cudaStream_t s) {
-  if (c->tangent) return launch3<lbmk::Dual>(c, c->ct, read, s);
-  return c->f64 ? launch3<double>(c, c->cd, read, s) : launch3<float>(c, c->cf, read, s);
+cudaError_t launch3(lbm3_ctx* c, const lbmn::ReadOut* ro, cudaStream_t s) {
+  if (c->tangent) return launch3<lbmk::Dual>(c, c->nt, ro, s);
+  return c->f64 ? launch3<double>(c, c->nd, ro, s) : launch3<float>(c, c->nf, ro, s);
+}
+
+// the read-out of the selected fields into the context's own planes
+lbmn::ReadOut own_planes(const lbm3_ctx* c, uint32_t mask) {
+  lbmn::ReadOut ro;
+  std::memset(&ro, 0, sizeof(ro));
+  const size_t N = (size_t)c->g.nx * c->g.ny * c->g.nz;
+  for (int k = 0; k < lbm3::NFIELD3; k++)
+    if (mask >> k & 1u) ro.out[k] = c->fld + k * N;
+  return ro;
 }
 
 template <typename R>
@@ -876,6 +622,21 @@ int lbm3_create(const lbm3_params* p, lbm3_ctx** out) {
   c->cf = lbmh::make_coef<float>(p->base);
   c->cd = lbmh::make_coef<double>(p->base);
   if (c->tangent) c->ct = lbmh::make_coef_tangent(p->base);
+  {
+    const double g[3] = {p->base.gx, p->base.gy, p->gz};
+    double T[6], dT[6];
+    for (int k = 0; k < 4; k++) {
+      T[k] = p->base.T_wall[k];
+      dT[k] = p->base.tan_T_wall[k];
+    }
+    for (int k = 0; k < 2; k++) {
+      T[4 + k] = p->T_wall_z[k];
+      dT[4 + k] = p->tan_T_wall_z[k];
+    }
+    c->nf = lbmh::make_node_coef<float, 3>(p->base, g, T, dT);
+    c->nd = lbmh::make_node_coef<double, 3>(p->base, g, T, dT);
+    c->nt = lbmh::make_node_coef<lbmk::Dual, 3>(p->base, g, T, dT);
+  }
   const size_t es = c->tangent ? 16 : (c->f64 ? 8 : 4);
   const size_t fmul = c->tangent ? 2 : 1;  // read-out and diagnostics: values, then derivatives
   const long long N = (long long)p->base.nx * p->base.ny * p->nz;
@@ -955,7 +716,7 @@ int lbm3_step(lbm3_ctx* c, int64_t nsteps, void* stream) {
   if (!c->have_geometry) return fail3(c, LBM_ERR_STATE, "step before lbm3_set_geometry");
   cudaStream_t s = (cudaStream_t)stream;
   for (int64_t k = 0; k < nsteps; k++) {
-    const cudaError_t e = launch3(c, false, s);
+    const cudaError_t e = launch3(c, nullptr, s);
     if (e != cudaSuccess) return cuda_fail3(c, e, "lbm3_step");
     c->cur ^= 1;
     c->step++;
@@ -973,8 +734,14 @@ int lbm3_read_fields(lbm3_ctx* c, uint32_t field_mask, double* const* out, int w
     if ((field_mask >> k & 1u) && !out[k]) return fail3(c, LBM_ERR_ARG, "null output for a selected field");
   cudaStream_t s = (cudaStream_t)stream;
   const size_t N = (size_t)c->g.nx * c->g.ny * c->g.nz;
-  cudaError_t e = launch3(c, true, s);
-  for (int k = 0; k < lbm3::NFIELD3 && e == cudaSuccess; k++)
+  // device outputs are written in place; host ones and a tangent's (whose
+  // derivatives come with the values) through the context's planes
+  const bool direct = where == LBM_DEVICE && !c->tangent;
+  lbmn::ReadOut ro = own_planes(c, field_mask);
+  for (int k = 0; k < lbm3::NFIELD3 && direct; k++)
+    if (field_mask >> k & 1u) ro.out[k] = out[k];
+  cudaError_t e = launch3(c, &ro, s);
+  for (int k = 0; k < lbm3::NFIELD3 && e == cudaSuccess && !direct; k++)
     if (field_mask >> k & 1u)
       e = cudaMemcpyAsync(out[k], c->fld + k * N, N * sizeof(double),
                           where == LBM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s);
@@ -994,7 +761,8 @@ int lbm3_read_tangent_fields(lbm3_ctx* c, uint32_t field_mask, double* const* ou
     if ((field_mask >> k & 1u) && !out[k]) return fail3(c, LBM_ERR_ARG, "null output for a selected field");
   cudaStream_t s = (cudaStream_t)stream;
   const size_t N = (size_t)c->g.nx * c->g.ny * c->g.nz;
-  cudaError_t e = launch3(c, true, s);
+  const lbmn::ReadOut ro = own_planes(c, field_mask);
+  cudaError_t e = launch3(c, &ro, s);
   for (int k = 0; k < lbm3::NFIELD3 && e == cudaSuccess; k++)
     if (field_mask >> k & 1u)
       e = cudaMemcpyAsync(out[k], c->fld + (lbm3::NFIELD3 + k) * N, N * sizeof(double),
@@ -1028,7 +796,8 @@ int lbm3_diagnostics(lbm3_ctx* c, lbm_diag* out, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   double h[2 * lbm3::NDIAG3];
   const size_t rows = c->tangent ? 2 * lbm3::NDIAG3 : lbm3::NDIAG3;
-  cudaError_t e = launch3(c, true, s);
+  const lbmn::ReadOut ro = own_planes(c, (1u << lbm3::NFIELD3) - 1);
+  cudaError_t e = launch3(c, &ro, s);
   if (e == cudaSuccess)
     e = c->tangent ? launch_diag3<lbmk::Dual>(c, c->ct, s)
         : c->f64   ? launch_diag3<double>(c, c->cd, s)

@@ -15,20 +15,20 @@ constexpr int min_blocks() {
 template <typename R, int LATC>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_local_kernel(const __grid_constant__ NodeArgs<R, 2> a) {
-  node_local<R, 2, LATC, int>(a, blockIdx.x * blockDim.x + threadIdx.x);
+  node_local_linear<R, 2, LATC, int>(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <typename R, int LATC, bool DIAG>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_collide_kernel(const __grid_constant__ NodeArgs<R, 2> a) {
-  node_collide<R, 2, LATC, false, DIAG, int>(a, nullptr, blockIdx.x * blockDim.x + threadIdx.x);
+  node_collide_linear<R, 2, LATC, false, DIAG, int>(a, nullptr, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <typename R, int LATC, bool DIAG>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_read_kernel(const __grid_constant__ NodeArgs<R, 2> a,
                      const __grid_constant__ ReadOut ro) {
-  node_collide<R, 2, LATC, true, DIAG, int>(a, &ro, blockIdx.x * blockDim.x + threadIdx.x);
+  node_collide_linear<R, 2, LATC, true, DIAG, int>(a, &ro, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Warps per block: four where that still gives every SM several blocks; a
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(NTN, 2)
     else hi = mid;
   }
   const int id = (t - B.base[lo]) * blockDim.x + threadIdx.x;
-  if (COLLIDE) node_collide<double, 2, LATC, false, DIAG, int>(B.args[lo], nullptr, id);
-  else node_local<double, 2, LATC, int>(B.args[lo], id);
+  if (COLLIDE) node_collide_linear<double, 2, LATC, false, DIAG, int>(B.args[lo], nullptr, id);
+  else node_local_linear<double, 2, LATC, int>(B.args[lo], id);
 }
 
 template <int LATC>

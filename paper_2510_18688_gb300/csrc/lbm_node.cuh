@@ -297,6 +297,20 @@ __device__ __forceinline__ Pos<D> node_pos(const NodeGeom<D>& g, int id) {
   p.n = row * g.pitch + p.x[0];
   return p;
 }
+// the node at (x, y, z), and its id in the dense order of the outputs
+__device__ __forceinline__ Pos<3> node_at(const NodeGeom<3>& g, int x, int y, int z) {
+  Pos<3> p;
+  p.x[0] = x;
+  p.x[1] = y;
+  p.x[2] = z;
+  p.n = (z * g.n[1] + y) * g.pitch + x;
+  return p;
+}
+template <int D>
+__device__ __forceinline__ long long dense_id(const NodeGeom<D>& g, const Pos<D>& p) {
+  if constexpr (D == 2) return (long long)p.x[1] * g.n[0] + p.x[0];
+  else return ((long long)p.x[2] * g.n[1] + p.x[1]) * g.n[0] + p.x[0];
+}
 
 // Offsets to the neighbours along each axis (wrapped on a periodic axis, 0
 // -- the node itself, mirrored -- beyond a wall) and the walls they lie
@@ -456,15 +470,13 @@ __device__ __forceinline__ LocalState<R> local_of(const NodeCoef<R, D>& c, int l
 
 // I: the type of plane offsets (int while all population planes fit 31 bits)
 template <typename R, int D, int LATC, typename I>
-__device__ __forceinline__ void node_local(const NodeArgs<R, D>& a, int id) {
+__device__ __forceinline__ void node_local(const NodeArgs<R, D>& a, int n) {
   const NodeGeom<D>& g = a.g;
   const NodeCoef<R, D>& c = a.c;
   constexpr int Q = Lat<D>::Q;
   using L_ = Lag<D>;
   const int lat = LATC ? LATC : g.lattices;
-  if (id >= g.nodes) return;
   const I P = (I)g.plane;
-  const int n = node_pos<D>(g, id).n;
   const K<R> phi0 = plain(a.phi0[n]);
   const R flp = a.lin[L_::FL * P + n], wp = a.lin[L_::W * P + n], Qp = a.lin[L_::Q * P + n];
   R sg = R(0), sh = R(0);
@@ -634,9 +646,10 @@ __device__ __forceinline__ void warp_diag(double* diag, int nwarps, int wid, con
 }
 
 // READ: the field read-out of the state instead of the step.  Every lane of
-// a warp calls it (the diagnostics are warp sums).
+// a warp calls it (the diagnostics are warp sums, of warp wid).
 template <typename R, int D, int LATC, bool READ, bool DIAG, typename I>
-__device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const ReadOut* ro, int id) {
+__device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const ReadOut* ro, bool valid,
+                                             const Pos<D>& pos, int wid) {
   const NodeGeom<D>& g = a.g;
   const NodeCoef<R, D>& c = a.c;
   using L_ = Lat<D>;
@@ -650,9 +663,8 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
 #pragma unroll
     for (int k = 0; k < 8; k++) dv[k] = R(0);
   }
-  if (id < g.nodes) {
+  if (valid) {
     const I P = (I)g.plane;
-    const Pos<D> pos = node_pos<D>(g, id);
     const int n = pos.n;
     const Nbr<D> nb = neighbours<D>(g, pos);
     const R* sc = a.sc + n;
@@ -761,7 +773,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
 
     if (READ) {
       const R vals2[12] = {phi, fs, fl, T, rhoH, pr, u[0], u[1], rho, mu, w, mdot};
-      const long long N = g.nodes;
+      const long long N = g.nodes, id = dense_id<D>(g, pos);
       if constexpr (D == 2) {
 #pragma unroll
         for (int k = 0; k < 12; k++)
@@ -957,7 +969,19 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
       a.lout[G_::Q * P + n] = CTm;
     }
   }
-  if (DIAG) warp_diag(a.diag, a.nwarps, id >> 5, dv, bad);
+  if constexpr (DIAG) warp_diag(a.diag, a.nwarps, wid, dv, bad);
+}
+
+// node ids linear over the grid
+template <typename R, int D, int LATC, typename I>
+__device__ __forceinline__ void node_local_linear(const NodeArgs<R, D>& a, int id) {
+  if (id < a.g.nodes) node_local<R, D, LATC, I>(a, node_pos<D>(a.g, id).n);
+}
+template <typename R, int D, int LATC, bool READ, bool DIAG, typename I>
+__device__ __forceinline__ void node_collide_linear(const NodeArgs<R, D>& a, const ReadOut* ro,
+                                                    int id) {
+  const bool valid = id < a.g.nodes;
+  node_collide<R, D, LATC, READ, DIAG, I>(a, ro, valid, node_pos<D>(a.g, valid ? id : 0), id >> 5);
 }
 
 }  // namespace lbmn

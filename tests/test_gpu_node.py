@@ -140,6 +140,39 @@ def test_coupled_adjoint_with_all_states_equals_checkpoints(env, nx, ny, every, 
     b.close()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny,nz", [(31, 4, 3), (32, 4, 2), (33, 5, 4), (64, 2, 3), (5, 43, 6)])
+@pytest.mark.parametrize("seed", [0, 3])
+def test_three_dimensional_sizes_match_the_oracle(env, nx, ny, nz, seed):
+    """Grids around the float kernels' 32 x 4 x 2 blocks and the double ones'
+    128 linear nodes: FP64 at its parity bar, FP32 at 1e-4 in relative L2 (or
+    1e-6 of the field's scale), device and host read-outs alike."""
+    import torch
+    from oracle import oracle3d as O3
+    _, lbm = env
+    O3.build()
+    cfg, arr = W.random_state3(nx, ny, nz, seed=seed)
+    ref = O3.from_workload((cfg, arr)).step(15).fields()
+    for prec in ("fp64", "fp32"):
+        s = lbm.Solver3(cfg, prec).set_geometry(arr).step(15)
+        got = s.fields()
+        out = torch.full((13, nz, ny, nx), -7.0, dtype=torch.float64, device="cuda")
+        lbm.lbm3_read_fields(s.ctx, 0b1010000000101, [out[k].data_ptr() for k in range(13)],
+                             lbm.LBM_DEVICE, lbm._stream())
+        for i, k in enumerate(lbm.FIELDS3):
+            a, b = ref[k], got[k]
+            scale = max(np.abs(a).max(), 1e-30)
+            if prec == "fp64":
+                assert np.abs(a - b).max() <= 1e-10 * scale, k
+            else:
+                den = max(np.linalg.norm(a), 1e-30 * np.sqrt(a.size))
+                assert np.linalg.norm(a - b) <= 1e-4 * den or \
+                    np.abs(a - b).max() <= 1e-6 * max(scale, 1e-3), k
+            want = b if 0b1010000000101 >> i & 1 else np.full_like(b, -7.0)
+            assert np.array_equal(out[i].cpu().numpy(), want), k
+        s.close()
+
+
 def _fma(a, b, c):
     return float(Fraction(a) * Fraction(b) + Fraction(c))  # one rounding, as the device's fma
 
