@@ -170,6 +170,7 @@ constexpr int min_blocks() {
 template <typename R, typename I>
 __global__ void __launch_bounds__(kThreads<R>)
     lbm3_local_kernel(const __grid_constant__ lbmn::NodeArgs<R, 3> a) {
+  lbmk::after_previous();
   if constexpr (kTiled<R>) {
     const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
     const int z = blockIdx.z * BZ + threadIdx.z;
@@ -182,6 +183,7 @@ __global__ void __launch_bounds__(kThreads<R>)
 
 template <typename R, bool READ, typename I>
 __device__ __forceinline__ void collide3(const lbmn::NodeArgs<R, 3>& a, const lbmn::ReadOut* ro) {
+  lbmk::after_previous();
   if constexpr (kTiled<R>) {
     const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
     const int z = blockIdx.z * BZ + threadIdx.z;
@@ -520,9 +522,9 @@ lbmn::NodeArgs<R, 3> node_args3(lbm3_ctx* c, const lbmn::NodeCoef<R, 3>& coef) {
 template <typename R, typename I>
 void launch_step3(const lbmn::NodeArgs<R, 3>& a, const lbmn::ReadOut* ro, dim3 gd, dim3 bd,
                   cudaStream_t s) {
-  lbm3::lbm3_local_kernel<R, I><<<gd, bd, 0, s>>>(a);
-  if (ro) lbm3::lbm3_read_kernel<R, I><<<gd, bd, 0, s>>>(a, *ro);
-  else lbm3::lbm3_collide_kernel<R, I><<<gd, bd, 0, s>>>(a);
+  lbmk::launch_dep(lbm3::lbm3_local_kernel<R, I>, gd, bd, 0, s, a);
+  if (ro) lbmk::launch_dep(lbm3::lbm3_read_kernel<R, I>, gd, bd, 0, s, a, *ro);
+  else lbmk::launch_dep(lbm3::lbm3_collide_kernel<R, I>, gd, bd, 0, s, a);
 }
 
 template <typename R>

@@ -90,8 +90,8 @@ namespace lbmn {
 static int rev_blocks(const RevArgs& a) { return (a.f.g.nodes + REV_NT - 1) / REV_NT; }
 
 cudaError_t launch_rev_step(const RevArgs& a, cudaStream_t s) {
-  rev_collide_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a);
-  rev_local_kernel<<<rev_blocks(a), REV_NT, 0, s>>>(a);
+  lbmk::launch_dep(rev_collide_kernel, rev_blocks(a), REV_NT, 0, s, a);
+  lbmk::launch_dep(rev_local_kernel, rev_blocks(a), REV_NT, 0, s, a);
   return cudaGetLastError();
 }
 

@@ -91,6 +91,7 @@ static __global__ void __launch_bounds__(REV_NT, 6) rev_collide_kernel(const Rev
   const NodeCoef<double, 2>& c = a.f.c;
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= g.nodes) return;
+  lbmk::after_previous();
   const int P = (int)g.plane;
   const Pos<2> pos = node_pos<2>(g, id);
   const int n = pos.n;
@@ -270,6 +271,7 @@ static __global__ void __launch_bounds__(REV_NT, 6) rev_collide_kernel(const Rev
 #pragma unroll
     for (int i = 1; i < 9; i++) lam[(18 + i) * P] = am * hb[Lat<2>::opp(i)];
   }
+  lbmk::allow_next();
   // ---- pressure Eq. (17c), tau_f, forces, velocity ------------------------------------
   {
     const double pk = prb * (1.0 / (3.0 * (1.0 - w0)));  // adjoint of sum_{i>0} f_i
@@ -369,6 +371,7 @@ static __global__ void __launch_bounds__(REV_NT, 8) rev_local_kernel(const RevAr
   const NodeCoef<double, 2>& c = a.f.c;
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= g.nodes) return;
+  lbmk::after_previous();
   const int P = (int)g.plane;
   const Pos<2> pos = node_pos<2>(g, id);
   const int n = pos.n;
@@ -452,6 +455,7 @@ static __global__ void __launch_bounds__(REV_NT, 8) rev_local_kernel(const RevAr
   double wpb = mr * (flp - fl);
   const double flpb = mr * wp;
   flb -= flpb;
+  lbmk::allow_next();
   // the inversion of Eq. (8)
   const double ell = wp * c.rl;
   const bool frozen = rhoH < 0.0, liquid = rhoH > ell && !frozen;

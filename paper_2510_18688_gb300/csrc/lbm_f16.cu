@@ -9,9 +9,9 @@ static void launch_one(const Args<float, __half>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    lbm_step_kernel<float, MODE, DIAG, 7, __half, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, __half, TYS>, grid, block, 0, s, a);
   else
-    lbm_step_kernel<float, MODE, DIAG, 0, __half, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, __half, TYS>, grid, block, 0, s, a);
 }
 
 template <bool DIAG>
@@ -68,11 +68,11 @@ static void tile_launch(const TileArgs<__half>& t, bool diag, int grid, cudaStre
   const size_t smem = tile_smem_bytes<__half>(NST);
   const bool all = t.a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT);
   if (all) {
-    if (diag) lbm_tile_kernel<__half, true, 7, NST><<<grid, block_dims(), smem, s>>>(t);
-    else lbm_tile_kernel<__half, false, 7, NST><<<grid, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile_kernel<__half, true, 7, NST>, grid, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile_kernel<__half, false, 7, NST>, grid, block_dims(), smem, s, t);
   } else {
-    if (diag) lbm_tile_kernel<__half, true, 0, NST><<<grid, block_dims(), smem, s>>>(t);
-    else lbm_tile_kernel<__half, false, 0, NST><<<grid, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile_kernel<__half, true, 0, NST>, grid, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile_kernel<__half, false, 0, NST>, grid, block_dims(), smem, s, t);
   }
 }
 
@@ -101,11 +101,11 @@ static cudaError_t prepare_tile1() {
 static void tile1_launch(const TileArgs<__half>& t, bool diag, cudaStream_t s) {
   const size_t smem = tile_smem_bytes<__half>(1);
   if (t.a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT)) {
-    if (diag) lbm_tile1_kernel<__half, true, 7><<<t.ntiles, block_dims(), smem, s>>>(t);
-    else lbm_tile1_kernel<__half, false, 7><<<t.ntiles, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile1_kernel<__half, true, 7>, t.ntiles, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile1_kernel<__half, false, 7>, t.ntiles, block_dims(), smem, s, t);
   } else {
-    if (diag) lbm_tile1_kernel<__half, true, 0><<<t.ntiles, block_dims(), smem, s>>>(t);
-    else lbm_tile1_kernel<__half, false, 0><<<t.ntiles, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile1_kernel<__half, true, 0>, t.ntiles, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile1_kernel<__half, false, 0>, t.ntiles, block_dims(), smem, s, t);
   }
 }
 

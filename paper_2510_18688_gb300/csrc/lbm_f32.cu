@@ -9,9 +9,9 @@ static void launch_one(const Args<float>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    lbm_step_kernel<float, MODE, DIAG, 7, float, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, float, TYS>, grid, block, 0, s, a);
   else
-    lbm_step_kernel<float, MODE, DIAG, 0, float, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, float, TYS>, grid, block, 0, s, a);
 }
 
 template <bool DIAG>
@@ -36,11 +36,11 @@ cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, cu
   const dim3 block = block_dims();
   const int ctas = b.tile_base[b.ngrids];
   if (all) {
-    if (diag) lbm_batch_kernel<float, true, 7><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<float, false, 7><<<ctas, block, 0, s>>>(b);
+    if (diag) launch_dep(lbm_batch_kernel<float, true, 7>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<float, false, 7>, ctas, block, 0, s, b);
   } else {
-    if (diag) lbm_batch_kernel<float, true, 0><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<float, false, 0><<<ctas, block, 0, s>>>(b);
+    if (diag) launch_dep(lbm_batch_kernel<float, true, 0>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<float, false, 0>, ctas, block, 0, s, b);
   }
   return cudaGetLastError();
 }
@@ -92,11 +92,11 @@ static void tile_launch(const TileArgs<float>& t, bool diag, int grid, cudaStrea
   const size_t smem = tile_smem_bytes<float>(NST);
   const bool all = t.a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT);
   if (all) {
-    if (diag) lbm_tile_kernel<float, true, 7, NST><<<grid, block_dims(), smem, s>>>(t);
-    else lbm_tile_kernel<float, false, 7, NST><<<grid, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile_kernel<float, true, 7, NST>, grid, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile_kernel<float, false, 7, NST>, grid, block_dims(), smem, s, t);
   } else {
-    if (diag) lbm_tile_kernel<float, true, 0, NST><<<grid, block_dims(), smem, s>>>(t);
-    else lbm_tile_kernel<float, false, 0, NST><<<grid, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile_kernel<float, true, 0, NST>, grid, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile_kernel<float, false, 0, NST>, grid, block_dims(), smem, s, t);
   }
 }
 
@@ -125,11 +125,11 @@ static cudaError_t prepare_tile1() {
 static void tile1_launch(const TileArgs<float>& t, bool diag, cudaStream_t s) {
   const size_t smem = tile_smem_bytes<float>(1);
   if (t.a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT)) {
-    if (diag) lbm_tile1_kernel<float, true, 7><<<t.ntiles, block_dims(), smem, s>>>(t);
-    else lbm_tile1_kernel<float, false, 7><<<t.ntiles, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile1_kernel<float, true, 7>, t.ntiles, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile1_kernel<float, false, 7>, t.ntiles, block_dims(), smem, s, t);
   } else {
-    if (diag) lbm_tile1_kernel<float, true, 0><<<t.ntiles, block_dims(), smem, s>>>(t);
-    else lbm_tile1_kernel<float, false, 0><<<t.ntiles, block_dims(), smem, s>>>(t);
+    if (diag) launch_dep(lbm_tile1_kernel<float, true, 0>, t.ntiles, block_dims(), smem, s, t);
+    else launch_dep(lbm_tile1_kernel<float, false, 0>, t.ntiles, block_dims(), smem, s, t);
   }
 }
 
@@ -144,11 +144,11 @@ cudaError_t launch_tile_batch_f32(const TileBatch<float>& b, bool diag, bool all
   const size_t smem = tile_smem_bytes<float>(1);
   const int ctas = b.tile_base[b.ngrids];
   if (all) {
-    if (diag) lbm_tile_batch_kernel<float, true, 7><<<ctas, block_dims(), smem, s>>>(b);
-    else lbm_tile_batch_kernel<float, false, 7><<<ctas, block_dims(), smem, s>>>(b);
+    if (diag) launch_dep(lbm_tile_batch_kernel<float, true, 7>, ctas, block_dims(), smem, s, b);
+    else launch_dep(lbm_tile_batch_kernel<float, false, 7>, ctas, block_dims(), smem, s, b);
   } else {
-    if (diag) lbm_tile_batch_kernel<float, true, 0><<<ctas, block_dims(), smem, s>>>(b);
-    else lbm_tile_batch_kernel<float, false, 0><<<ctas, block_dims(), smem, s>>>(b);
+    if (diag) launch_dep(lbm_tile_batch_kernel<float, true, 0>, ctas, block_dims(), smem, s, b);
+    else launch_dep(lbm_tile_batch_kernel<float, false, 0>, ctas, block_dims(), smem, s, b);
   }
   return cudaGetLastError();
 }

@@ -10,9 +10,9 @@ static void launch_one(const Args<double>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    lbm_step_kernel<double, MODE, DIAG, 7, double, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<double, MODE, DIAG, 7, double, TYS>, grid, block, 0, s, a);
   else
-    lbm_step_kernel<double, MODE, DIAG, 0, double, TYS><<<grid, block, 0, s>>>(a);
+    launch_dep(lbm_step_kernel<double, MODE, DIAG, 0, double, TYS>, grid, block, 0, s, a);
 }
 
 template <bool DIAG>
@@ -37,17 +37,17 @@ cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, c
   const dim3 block = block_dims(THIN_TY);
   const int ctas = b.tile_base[b.ngrids];
   if (all) {
-    if (diag) lbm_batch_kernel<double, true, 7, THIN_TY><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<double, false, 7, THIN_TY><<<ctas, block, 0, s>>>(b);
+    if (diag) launch_dep(lbm_batch_kernel<double, true, 7, THIN_TY>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<double, false, 7, THIN_TY>, ctas, block, 0, s, b);
   } else {
-    if (diag) lbm_batch_kernel<double, true, 0, THIN_TY><<<ctas, block, 0, s>>>(b);
-    else lbm_batch_kernel<double, false, 0, THIN_TY><<<ctas, block, 0, s>>>(b);
+    if (diag) launch_dep(lbm_batch_kernel<double, true, 0, THIN_TY>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<double, false, 0, THIN_TY>, ctas, block, 0, s, b);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_diag_f64(const Args<double>& a, cudaStream_t s) {
-  lbm_step_kernel<double, MODE_READ, true, 0><<<grid_dims(a.g), block_dims(), 0, s>>>(a);
+  launch_dep(lbm_step_kernel<double, MODE_READ, true, 0>, grid_dims(a.g), block_dims(), 0, s, a);
   return cudaGetLastError();
 }
 

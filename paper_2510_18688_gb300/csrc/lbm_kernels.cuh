@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_dual.cuh"
+#include "lbm_pdl.cuh"
 
 namespace lbmk {
 

@@ -15,12 +15,14 @@ constexpr int min_blocks() {
 template <typename R, int LATC>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_local_kernel(const __grid_constant__ NodeArgs<R, 2> a) {
+  lbmk::after_previous();
   node_local_linear<R, 2, LATC, int>(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 template <typename R, int LATC, bool DIAG>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_collide_kernel(const __grid_constant__ NodeArgs<R, 2> a) {
+  lbmk::after_previous();
   node_collide_linear<R, 2, LATC, false, DIAG, int>(a, nullptr, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -28,6 +30,7 @@ template <typename R, int LATC, bool DIAG>
 __global__ void __launch_bounds__(NTN, min_blocks<R>())
     node_read_kernel(const __grid_constant__ NodeArgs<R, 2> a,
                      const __grid_constant__ ReadOut ro) {
+  lbmk::after_previous();
   node_collide_linear<R, 2, LATC, true, DIAG, int>(a, &ro, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -42,13 +45,13 @@ template <typename R, int LATC>
 static void launch_lat(const NodeArgs<R, 2>& a, const ReadOut* ro, bool diag, int wpb,
                        cudaStream_t s) {
   const int nt = 32 * wpb, nb = (a.nwarps + wpb - 1) / wpb;
-  node_local_kernel<R, LATC><<<nb, nt, 0, s>>>(a);
+  lbmk::launch_dep(node_local_kernel<R, LATC>, nb, nt, 0, s, a);
   if (ro) {
-    if (diag) node_read_kernel<R, LATC, true><<<nb, nt, 0, s>>>(a, *ro);
-    else node_read_kernel<R, LATC, false><<<nb, nt, 0, s>>>(a, *ro);
+    if (diag) lbmk::launch_dep(node_read_kernel<R, LATC, true>, nb, nt, 0, s, a, *ro);
+    else lbmk::launch_dep(node_read_kernel<R, LATC, false>, nb, nt, 0, s, a, *ro);
   } else {
-    if (diag) node_collide_kernel<R, LATC, true><<<nb, nt, 0, s>>>(a);
-    else node_collide_kernel<R, LATC, false><<<nb, nt, 0, s>>>(a);
+    if (diag) lbmk::launch_dep(node_collide_kernel<R, LATC, true>, nb, nt, 0, s, a);
+    else lbmk::launch_dep(node_collide_kernel<R, LATC, false>, nb, nt, 0, s, a);
   }
 }
 
@@ -66,8 +69,8 @@ template cudaError_t launch_node<Dual>(const NodeArgs<Dual, 2>&, const ReadOut*,
 
 cudaError_t launch_node_local(const NodeArgs<double, 2>& a, cudaStream_t s) {
   const int wpb = warps_per_block(a.nwarps), nt = 32 * wpb, nb = (a.nwarps + wpb - 1) / wpb;
-  if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT)) node_local_kernel<double, 7><<<nb, nt, 0, s>>>(a);
-  else node_local_kernel<double, 0><<<nb, nt, 0, s>>>(a);
+  if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT)) lbmk::launch_dep(node_local_kernel<double, 7>, nb, nt, 0, s, a);
+  else lbmk::launch_dep(node_local_kernel<double, 0>, nb, nt, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -85,6 +88,7 @@ __global__ void __launch_bounds__(NTN, 2)
     else hi = mid;
   }
   const int id = (t - B.base[lo]) * blockDim.x + threadIdx.x;
+  lbmk::after_previous();
   if (COLLIDE) node_collide_linear<double, 2, LATC, false, DIAG, int>(B.args[lo], nullptr, id);
   else node_local_linear<double, 2, LATC, int>(B.args[lo], id);
 }
@@ -92,9 +96,9 @@ __global__ void __launch_bounds__(NTN, 2)
 template <int LATC>
 static void launch_batch_lat(const NodeBatch& b, bool diag, cudaStream_t s) {
   const int nt = NODE_BATCH_THREADS, nb = b.base[b.ngrids];
-  node_batch_kernel<false, LATC, false><<<nb, nt, 0, s>>>(b);
-  if (diag) node_batch_kernel<true, LATC, true><<<nb, nt, 0, s>>>(b);
-  else node_batch_kernel<true, LATC, false><<<nb, nt, 0, s>>>(b);
+  lbmk::launch_dep(node_batch_kernel<false, LATC, false>, nb, nt, 0, s, b);
+  if (diag) lbmk::launch_dep(node_batch_kernel<true, LATC, true>, nb, nt, 0, s, b);
+  else lbmk::launch_dep(node_batch_kernel<true, LATC, false>, nb, nt, 0, s, b);
 }
 
 cudaError_t launch_node_batch(const NodeBatch& b, bool diag, bool all, cudaStream_t s) {

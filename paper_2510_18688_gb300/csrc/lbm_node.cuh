@@ -497,6 +497,7 @@ __device__ __forceinline__ void node_local(const NodeArgs<R, D>& a, int n) {
     sh = sum_pops<D, true>(v);
   }
   const LocalState<R> L = local_of<R, D>(c, lat, sg, sh, flp, wp, Qp, phi0);
+  lbmk::allow_next();
   R* sc = a.sc + n;
   sc[SC_PHI * P] = L.phi;
   sc[SC_CHI * P] = mad(L.fs, c.cos_ps, mad(c.cos_th, phi0, L.phi));
@@ -916,6 +917,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
         }
       }
 
+      lbmk::allow_next();
       // ---- enthalpy TRT collision Eqs. (23)-(27) --------------------------------
       R CTm = R(0);
       if (lat & LAT_HEAT) {

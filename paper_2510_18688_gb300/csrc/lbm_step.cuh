@@ -749,6 +749,7 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     for (int k = tid; k < RING; k += NT) ring_state(k);
   }
   __syncthreads();
+  if (MODE == MODE_STEP) allow_next();
 
   // ---- phase B: stencils, macros, collisions, streaming -------------------
   // Instantiated twice: for a tile whose nodes and ring are all inside the
@@ -883,6 +884,7 @@ template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = T
 __global__ void __launch_bounds__(Shape<TYS>::NT,
                                   sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 * TY / TYS : 1)
     lbm_step_kernel(const Args<R, S> a) {
+  after_previous();
   step_tile<R, MODE, DIAG, LATC, S, TYS>(a, blockIdx.x, blockIdx.y, -1, 0);
 }
 
@@ -905,6 +907,7 @@ struct BatchTable {
 template <typename R, bool DIAG, int LATC, int TYS = TY>
 __global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
     lbm_batch_kernel(const __grid_constant__ BatchTable<R> B) {
+  after_previous();
   const int t = blockIdx.x;
   int lo = 0, hi = B.ngrids;  // tile_base[lo] <= t < tile_base[hi]
   while (hi - lo > 1) {

@@ -270,6 +270,7 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
     s_T[hi] = Lq.T;
   }
   __syncthreads();
+  allow_next();
 
   // ---- phase B: stencils, macros, collisions, streaming -------------------
   // Instantiated twice: for a tile whose nodes and ring are all inside the
@@ -367,6 +368,7 @@ __global__ void __launch_bounds__(NT, tile_min_blocks<NST>())
     tma_prefetch_map(&ta.map_gh);
     tma_prefetch_map(&ta.map_lag);
   }
+  after_previous();
   __syncthreads();
   int t = blockIdx.x, k = 0;
   if (tid == 0 && t < ta.ntiles) tile_issue(ta, stage[0], &bar[0], t);
@@ -433,6 +435,9 @@ __device__ __forceinline__ void tile_once(const Args<float, S>& a, const CUtenso
   if (tid == 0) {
     mbar_init(&bar, 1);
     fence_barrier_init();
+  }
+  after_previous();
+  if (tid == 0) {
     tile_issue_maps(mf, mgh, mlag, mphi0, extra_tx, stage[0], &bar, bx * TX, by * TY);
   }
   __syncthreads();
