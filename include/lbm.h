@@ -281,7 +281,7 @@ void lbm_destroy(lbm_ctx* ctx);
  * results agree to the last bit where the compiler contracts both kernels'
  * copies of the arithmetic alike, as the FP64 build does, and otherwise to a
  * few roundings of the working precision).  LBM_FP64 batches take two launches
- * per step and per 64 grids, and one more per 64 grids of few rows.  This is how
+ * per step and per 64 grids, and one more per 64 columns.  This is how
  * many small problems fill the GPU.  LBM_FP32 batches run as the batched
  * TMA-staged tile kernel (each tile's inputs copied to shared memory by the
  * tensor copies of its own context, one CTA per 32 x 8 tile; a copy that
@@ -434,10 +434,10 @@ int lbm_adjoint_coupled(lbm_ctx* ctx, int64_t nsteps, int every, int observable,
  * and state and keeps the fastest for later lbm_step calls.  Variant v is
  * kernel form v / 2 with captured periods of at least 32 steps (v even) or
  * 256 (v odd).  Kernel forms (form ids; a context times those it has):
- * 0 float: one CTA per 32 x 8 tile loading from global memory, LBM_FP64 and
- * tangents: the default, two node kernels of one thread per node (LBM_FP64
- * grids of fewer than 32 rows and at most 32768 nodes: one CTA per 32 x 1
- * tile); 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one
+ * 0 float: as 1, on columns one CTA per 32 x 8 tile loading from global
+ * memory (LBM_STEP_KERNEL=fused: everywhere), LBM_FP64 and tangents: the default, two node kernels of one thread per node (LBM_FP64
+ * columns, fewer than 32 rows and at least four times as long: one CTA per
+ * 32 x 1 tile); 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one
  * shared-memory stage and one CTA per tile, LBM_FP64: the node kernels; 2 (float) the
  * TMA-staged kernel with two stages and two persistent CTAs per
  * multiprocessor (the copies of the next tile overlap the current one);

@@ -61,6 +61,7 @@ struct lbm_ctx {
   // float contexts: the step as the TMA-staged tile kernel (lbm_tile.cuh)
   bool tile;
   bool tile_ok;          // the tile kernel's tensor maps exist (float contexts)
+  bool tile0;            // form 0 is the tile kernel
   int form;              // kernel form (form_available, set_kernel_form)
   int ty;                // tile height of the one-CTA-per-tile step (4, 8 or 16)
   int tile_stages;       // shared-memory stages of the tile kernel (1 or 2)
@@ -68,7 +69,7 @@ struct lbm_ctx {
   int sms;               // multiprocessors of the context's device
   CUtensorMap tm_f[2], tm_gh[2], tm_lag[2], tm_phi0;  // per A/B buffer
   lbmk::TileMaps* d_maps;  // device copy of the maps by parity (FP32: for batches)
-  unsigned* status;      // device word: a tile's copies did not arrive in time
+  unsigned* status;      // pinned word a tile kernel sets when its copies did not arrive in time
   int cur;
   int64_t step;
   bool have_geometry;
@@ -85,10 +86,11 @@ struct lbm_ctx {
   cudaGraphExec_t graph;
   int graph_cur;         // buffer parity the graph starts from
   int64_t graph_phase;   // step index modulo the period it starts from
-  uint64_t gen;          // bumped when geometry or state is replaced
+  uint64_t gen;          // bumped when what captured steps hold changes, or the state is replaced
   uint64_t graph_gen;
   int graph_min;         // shortest captured period (32; lbm_autotune may change it)
   int graph_len;         // steps in the captured graph
+  int graph_hook;        // g_tile_timeout when it was captured
   // planes of lbm_adjoint_coupled, kept between calls up to kKeptWork bytes
   double* work;
   size_t work_len;       // doubles
@@ -224,12 +226,12 @@ void set_tile_config(lbm_ctx* c, int stages, int per_sm) {
   c->tile_grid = per_sm > 0 ? std::max(1, std::min(c->nblocks, per_sm * c->sms)) : c->nblocks;
 }
 
-// Kernel forms of the step (lbm_autotune).  Float: 0 one CTA per 32 x 8
-// tile; 1 TMA-staged, one stage, one CTA per tile; 2 TMA-staged, two stages,
+// Kernel forms of the step (lbm_autotune).  Float: 0 as 1, on columns one CTA
+// per 32 x 8 tile from global loads; 1 TMA-staged, one
+// stage, one CTA per tile; 2 TMA-staged, two stages,
 // two persistent CTAs per SM; 3 TMA-staged, one stage, three persistent CTAs
 // per SM; 4 one CTA per 32 x 4 tile; 5 one CTA per 32 x 16 tile.  FP64: 0
-// the node step, on grids of fewer than 32 rows one CTA per 32 x 1 tile; 1
-// the node step; 4 one CTA per 32 x 4 tile; 5 one CTA per 32 x 2 tile.
+// the node step, on columns one CTA per 32 x 1 tile; 1 the node step; 4 one CTA per 32 x 4 tile; 5 one CTA per 32 x 2 tile.
 // Tangent contexts: 0, the node step.
 bool form_available(const lbm_ctx* c, int form) {
   if (form < 0 || form >= kForms) return false;
@@ -253,22 +255,23 @@ void set_kernel_form(lbm_ctx* c, int form) {
     c->node = form == 1 || (form == 0 && c->node0);
     return;
   }
-  c->tile = c->tile_ok && form >= 1 && form <= 3;
-  if (form == 1) set_tile_config(c, 1, 0);
+  c->tile = c->tile_ok && ((form >= 1 && form <= 3) || (form == 0 && c->tile0));
+  if (form == 1 || form == 0) set_tile_config(c, 1, 0);
   else if (form == 2) set_tile_config(c, 2, 2);
   else if (form == 3) set_tile_config(c, 1, 3);
 }
 
 // A tile kernel whose copies did not arrive within its bounded wait sets
-// c->status; the next synchronising read reports it (once).
+// *c->status (pinned host memory: no copy to read it); the next synchronising
+// read, and every read of a float context's fields, reports it (once).  The
+// kernels of double and tangent contexts wait for no copies.
 int check_timeout(lbm_ctx* c, cudaStream_t s) {
-  if (!c->status) return LBM_OK;
-  unsigned v = 0;
-  cudaError_t e = cudaMemcpyAsync(&v, c->status, sizeof(v), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "status download");
-  if (v) {
-    cudaMemsetAsync(c->status, 0, sizeof(unsigned), s);
+  if (!c->tile_ok) return LBM_OK;
+  const cudaError_t e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(c, e, "synchronisation");
+  volatile unsigned* v = c->status;
+  if (*v) {
+    *v = 0;
     return fail(c, LBM_ERR_TIMEOUT,
                 "a step's tile copies did not arrive in time; the state is undefined%s");
   }
@@ -430,7 +433,7 @@ cudaError_t step_launches(lbm_ctx* c, int64_t nsteps, cudaStream_t s) {
 cudaError_t step_graph(lbm_ctx* c, int period, cudaGraphExec_t* out) {
   const int64_t phase = c->step % period;
   if (c->graph && c->graph_cur == c->cur && c->graph_phase == phase && c->graph_gen == c->gen &&
-      c->graph_len == period) {
+      c->graph_len == period && c->graph_hook == g_tile_timeout.load()) {
     *out = c->graph;
     return cudaSuccess;
   }
@@ -469,6 +472,7 @@ cudaError_t step_graph(lbm_ctx* c, int period, cudaGraphExec_t* out) {
   c->graph_phase = phase;
   c->graph_gen = c->gen;
   c->graph_len = period;
+  c->graph_hook = g_tile_timeout.load();
   *out = c->graph;
   return cudaSuccess;
 }
@@ -478,7 +482,7 @@ void free_all(lbm_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   void* dev[] = {c->pop[0], c->pop[1], c->lag[0],     c->lag[1],    c->phi0,   c->mask,
                  c->diag_partial, c->diag_out, c->staging, c->in_stage,
-                 c->scratch, c->status, c->d_maps, c->work};
+                 c->scratch, c->d_maps, c->work};
   for (void* p : dev)
     if (p) cudaFree(p);
   if (c->h_diag) cudaFreeHost(c->h_diag);
@@ -534,8 +538,7 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
   c->g = lbmh::make_geom(*params);
   {
     c->node0 = c->tangent || (params->precision == LBM_FP64 &&
-                              (params->ny >= lbmk::THIN_ROWS ||
-                               (long long)params->nx * params->ny > lbmk::THIN_NODES));
+                              !lbmk::is_column(params->nx, params->ny));
     c->node = c->node0;
     // LBM_STEP_GRAPHS=0 launches every step on its own instead of
     // replaying captured periods
@@ -573,8 +576,15 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
     e = dev_malloc((void**)&c->diag_partial, dmul * lbmk::NDIAG * c->diag_cap * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc((void**)&c->diag_out, dmul * (lbmk::NDIAG + 1) * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(c->mask, 0, P);
-  if (e == cudaSuccess) e = dev_malloc((void**)&c->status, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(unsigned));
+  if (e == cudaSuccess) {
+    // the diagnostics' host copy and, after it, the status word
+    const size_t nd = dmul * (lbmk::NDIAG + 1);
+    e = host_alloc((void**)&c->h_diag, (nd + 1) * sizeof(double));
+    if (e == cudaSuccess) {
+      c->status = (unsigned*)(c->h_diag + nd);
+      *c->status = 0;
+    }
+  }
   if (e == cudaSuccess && (params->precision == LBM_FP32 || params->precision == LBM_FP16S)) {
     // the TMA-staged tile kernel needs its tensor maps and shared-memory sizes
     const bool maps = params->precision == LBM_FP32
@@ -599,13 +609,15 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
       e = dev_malloc((void**)&c->d_maps, sizeof(hm));
       if (e == cudaSuccess) e = cudaMemcpy(c->d_maps, hm, sizeof(hm), cudaMemcpyHostToDevice);
     }
-    // Default kernel form (lbm_autotune measures them all): one CTA per
-    // tile from global loads on grids of fewer than eight tiles per
-    // multiprocessor, where every tile's loads and compute overlap with
-    // the other resident CTAs'; the TMA-staged form with one CTA per tile on
-    // larger grids.  LBM_STEP_KERNEL=fused forces the first,
-    // LBM_TILE=<stages>:<CTAs per SM> (0: one CTA per tile) a tile kernel.
-    int form = (c->tile_ok && c->nblocks >= 8 * c->sms) ? 1 : 0;
+    // Default kernel form (lbm_autotune measures them all): the TMA-staged
+    // form with one CTA per tile (512 x 512: 17 us a step against 22 us from
+    // global loads, 2048 x 1024: 106 against 144), but for columns (is_column).
+    // LBM_STEP_KERNEL=fused forces global loads, LBM_TILE=<stages>:<CTAs per
+    // SM> (0: one CTA per tile) a tile kernel.
+    c->tile0 = c->tile_ok && !lbmk::is_column(params->nx, params->ny);
+    if (const char* k = std::getenv("LBM_STEP_KERNEL"))
+      if (std::strcmp(k, "fused") == 0) c->tile0 = false;
+    int form = 0;
     if (const char* v = std::getenv("LBM_TILE")) {
       int a = 0, b = 0;
       if (c->tile_ok && std::sscanf(v, "%d:%d", &a, &b) == 2 && (a == 1 || a == 2) && b >= 0 &&
@@ -625,8 +637,6 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
     const long v = std::strtol(f, &end, 10);
     if (end != f && form_available(c, (int)v)) set_kernel_form(c, (int)v);
   }
-  if (e == cudaSuccess)
-    e = host_alloc((void**)&c->h_diag, dmul * (lbmk::NDIAG + 1) * sizeof(double));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     int code = cuda_fail(c, e, "lbm_create allocation");
@@ -681,6 +691,9 @@ int lbm_set_geometry(lbm_ctx* c, const double* phi0, const uint8_t* cold_mask,
       d_mask = mb;
     }
   }
+  // captured steps hold pointers, constants and whether there is a mask: they
+  // serve the new geometry too unless the last changed
+  if (c->g.has_mask != (cold_mask ? 1 : 0)) c->gen++;
   c->g.has_mask = cold_mask ? 1 : 0;
   c->cur = 0;
   if (c->p.precision == LBM_FP32) {
@@ -719,7 +732,6 @@ int lbm_set_geometry(lbm_ctx* c, const double* phi0, const uint8_t* cold_mask,
     if (e != cudaSuccess) return cuda_fail(c, e, "set_geometry synchronisation");
   }
   c->step = 0;
-  c->gen++;  // captured steps of the old geometry are stale
   c->have_geometry = true;
   c->have_diag = false;
   c->diag_pending = false;
@@ -1872,11 +1884,12 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, void* stream, doubl
 struct lbm_batch {
   std::vector<lbm_ctx*> ctx;
   int precision;
-  // argument tables of the batch's kernels: FP64 the node step and, for grids
-  // of few rows, one CTA per 32 x 1 tile (the contexts of each in `nodes` and
-  // `thin`); FP32 the batched TMA-staged tile kernel (one stage, one CTA per
-  // tile) or, with LBM_BATCH_KERNEL=fused, one CTA per tile from global memory
-  std::vector<lbm_ctx*> nodes, thin;
+  // argument tables of the batch's kernels: FP64 the node step, FP32 the
+  // batched TMA-staged tile kernel (`tile`; one stage, one CTA per tile) or,
+  // with LBM_BATCH_KERNEL=fused, one CTA per tile from global memory, as the
+  // columns take in either precision.  The contexts of each: `wide`, `thin`.
+  std::vector<lbm_ctx*> wide, thin;
+  bool tile;
   lbmn::NodeBatch* ntab;
   lbmk::BatchTable<double>* dtab;
   lbmk::TileBatch<float>* ttab;
@@ -1960,7 +1973,7 @@ void note_batch_diag(lbm_batch* b, int64_t first0, int64_t n) {
 }
 
 // One step of a list of contexts by the kernel `kind` of their group.
-enum { BATCH_NODE, BATCH_THIN, BATCH_TILE, BATCH_FUSED };
+enum { BATCH_NODE, BATCH_THIN, BATCH_TILE, BATCH_FUSED, BATCH_COLUMN };
 cudaError_t batch_group(lbm_batch* b, const std::vector<lbm_ctx*>& list, int kind, bool diag,
                         cudaStream_t s) {
   static_assert(lbmn::NODE_BATCH_GRIDS == lbmk::BATCH_MAX_GRIDS, "one chunk size for all tables");
@@ -1980,7 +1993,7 @@ cudaError_t batch_group(lbm_batch* b, const std::vector<lbm_ctx*>& list, int kin
       e = lbmk::launch_tile_batch_f32(*b->ttab, diag, all, s);
     } else {
       const bool all = fill_table(ctx, count, *b->ftab, lbmk::TY);
-      e = lbmk::launch_batch_f32(*b->ftab, diag, all, s);
+      e = lbmk::launch_batch_f32(*b->ftab, diag, all, kind == BATCH_COLUMN, s);
     }
     if (e != cudaSuccess) return e;
   }
@@ -1991,14 +2004,11 @@ cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
   lbm_ctx* c0 = b->ctx[0];
   for (int64_t k = 0; k < nsteps; k++) {
     const bool diag = c0->p.diag_every > 0 && (c0->step % c0->p.diag_every) == 0;
-    cudaError_t e;
-    if (b->precision == LBM_FP64) {
-      // each grid by its own default kernel, as lbm_step takes it
-      e = batch_group(b, b->nodes, BATCH_NODE, diag, s);
-      if (e == cudaSuccess) e = batch_group(b, b->thin, BATCH_THIN, diag, s);
-    } else {
-      e = batch_group(b, b->ctx, b->ttab ? BATCH_TILE : BATCH_FUSED, diag, s);
-    }
+    // each grid by its own default kernel, as lbm_step takes it
+    const bool f64 = b->precision == LBM_FP64;
+    cudaError_t e =
+        batch_group(b, b->wide, f64 ? BATCH_NODE : (b->tile ? BATCH_TILE : BATCH_FUSED), diag, s);
+    if (e == cudaSuccess) e = batch_group(b, b->thin, f64 ? BATCH_THIN : BATCH_COLUMN, diag, s);
     if (e != cudaSuccess) return e;
     note_batch_diag(b, c0->step, 1);
     for (lbm_ctx* c : b->ctx) {
@@ -2018,6 +2028,7 @@ std::vector<uint64_t> batch_key(const lbm_batch* b, int period) {
   }
   k.push_back((uint64_t)(b->ctx[0]->step % period));
   k.push_back((uint64_t)period);
+  k.push_back((uint64_t)g_tile_timeout.load());
   return k;
 }
 
@@ -2121,19 +2132,24 @@ int lbm_batch_create(lbm_ctx* const* ctxs, int count, lbm_batch** out) {
   if (!b) return LBM_ERR_OOM;
   b->ctx.assign(ctxs, ctxs + count);
   b->precision = ctxs[0]->p.precision;
-  if (b->precision == LBM_FP64) {
-    for (lbm_ctx* c : b->ctx) (c->node0 ? b->nodes : b->thin).push_back(c);
+  const bool f64 = b->precision == LBM_FP64;
+  const char* k = std::getenv("LBM_BATCH_KERNEL");
+  b->tile = !(k && std::strcmp(k, "fused") == 0);
+  for (lbm_ctx* c : b->ctx) {
+    b->tile = b->tile && c->tile_ok && c->d_maps;
+    (lbmk::is_column(c->p.nx, c->p.ny) ? b->thin : b->wide).push_back(c);
+  }
+  bool ok = true;
+  if (f64) {
     b->ntab = new (std::nothrow) lbmn::NodeBatch();
     b->dtab = new (std::nothrow) lbmk::BatchTable<double>();
+    ok = b->ntab && b->dtab;
   } else {
-    bool tile = true;
-    for (int i = 0; i < count; i++) tile = tile && ctxs[i]->tile_ok && ctxs[i]->d_maps;
-    if (const char* k = std::getenv("LBM_BATCH_KERNEL"))
-      if (std::strcmp(k, "fused") == 0) tile = false;
-    if (tile) b->ttab = new (std::nothrow) lbmk::TileBatch<float>();
-    else b->ftab = new (std::nothrow) lbmk::BatchTable<float>();
+    b->ttab = new (std::nothrow) lbmk::TileBatch<float>();
+    b->ftab = new (std::nothrow) lbmk::BatchTable<float>();
+    ok = b->ttab && b->ftab;
   }
-  if (b->precision == LBM_FP64 ? !(b->ntab && b->dtab) : !(b->ttab || b->ftab)) {
+  if (!ok) {
     lbm_batch_destroy(b);
     return LBM_ERR_OOM;
   }

@@ -4,21 +4,23 @@
 
 namespace lbmk {
 
-template <int MODE, bool DIAG, int TYS = TY>
+// FEW: phase B in the form of lbm_wb.cuh (every grid but the columns)
+template <int MODE, bool DIAG, int TYS, bool FEW>
 static void launch_one(const Args<float, __half>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, __half, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, __half, TYS, FEW>, grid, block, 0, s, a);
   else
-    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, __half, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, __half, TYS, FEW>, grid, block, 0, s, a);
 }
 
 template <bool DIAG>
 static void launch_shape(const Args<float, __half>& a, int ty, cudaStream_t s) {
-  if (ty == 4) launch_one<MODE_STEP, DIAG, 4>(a, s);
-  else if (ty == 16) launch_one<MODE_STEP, DIAG, 16>(a, s);
-  else launch_one<MODE_STEP, DIAG>(a, s);
+  if (ty == 4) launch_one<MODE_STEP, DIAG, 4, true>(a, s);
+  else if (ty == 16) launch_one<MODE_STEP, DIAG, 16, true>(a, s);
+  else if (is_column(a.g.nx, a.g.ny)) launch_one<MODE_STEP, DIAG, TY, false>(a, s);
+  else launch_one<MODE_STEP, DIAG, TY, true>(a, s);
 }
 
 cudaError_t launch_step_f16s(const Args<float, __half>& a, int mode, bool diag, cudaStream_t s, int ty) {
@@ -26,8 +28,8 @@ cudaError_t launch_step_f16s(const Args<float, __half>& a, int mode, bool diag, 
     if (diag) launch_shape<true>(a, ty, s);
     else launch_shape<false>(a, ty, s);
   } else {
-    if (diag) launch_one<MODE_READ, true>(a, s);
-    else launch_one<MODE_READ, false>(a, s);
+    if (diag) launch_one<MODE_READ, true, TY, false>(a, s);
+    else launch_one<MODE_READ, false, TY, false>(a, s);
   }
   return cudaGetLastError();
 }

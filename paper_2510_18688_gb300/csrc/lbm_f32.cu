@@ -4,21 +4,23 @@
 
 namespace lbmk {
 
-template <int MODE, bool DIAG, int TYS = TY>
+// FEW: phase B in the form of lbm_wb.cuh (every grid but the columns)
+template <int MODE, bool DIAG, int TYS, bool FEW>
 static void launch_one(const Args<float>& a, cudaStream_t s) {
   const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, float, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 7, float, TYS, FEW>, grid, block, 0, s, a);
   else
-    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, float, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<float, MODE, DIAG, 0, float, TYS, FEW>, grid, block, 0, s, a);
 }
 
 template <bool DIAG>
 static void launch_shape(const Args<float>& a, int ty, cudaStream_t s) {
-  if (ty == 4) launch_one<MODE_STEP, DIAG, 4>(a, s);
-  else if (ty == 16) launch_one<MODE_STEP, DIAG, 16>(a, s);
-  else launch_one<MODE_STEP, DIAG>(a, s);
+  if (ty == 4) launch_one<MODE_STEP, DIAG, 4, true>(a, s);
+  else if (ty == 16) launch_one<MODE_STEP, DIAG, 16, true>(a, s);
+  else if (is_column(a.g.nx, a.g.ny)) launch_one<MODE_STEP, DIAG, TY, false>(a, s);
+  else launch_one<MODE_STEP, DIAG, TY, true>(a, s);
 }
 
 cudaError_t launch_step_f32(const Args<float>& a, int mode, bool diag, cudaStream_t s, int ty) {
@@ -26,22 +28,29 @@ cudaError_t launch_step_f32(const Args<float>& a, int mode, bool diag, cudaStrea
     if (diag) launch_shape<true>(a, ty, s);
     else launch_shape<false>(a, ty, s);
   } else {
-    if (diag) launch_one<MODE_READ, true>(a, s);
-    else launch_one<MODE_READ, false>(a, s);
+    if (diag) launch_one<MODE_READ, true, TY, false>(a, s);
+    else launch_one<MODE_READ, false, TY, false>(a, s);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, cudaStream_t s) {
+template <bool FEW>
+static void launch_batch_few(const BatchTable<float>& b, bool diag, bool all, cudaStream_t s) {
   const dim3 block = block_dims();
   const int ctas = b.tile_base[b.ngrids];
   if (all) {
-    if (diag) launch_dep(lbm_batch_kernel<float, true, 7>, ctas, block, 0, s, b);
-    else launch_dep(lbm_batch_kernel<float, false, 7>, ctas, block, 0, s, b);
+    if (diag) launch_dep(lbm_batch_kernel<float, true, 7, TY, FEW>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<float, false, 7, TY, FEW>, ctas, block, 0, s, b);
   } else {
-    if (diag) launch_dep(lbm_batch_kernel<float, true, 0>, ctas, block, 0, s, b);
-    else launch_dep(lbm_batch_kernel<float, false, 0>, ctas, block, 0, s, b);
+    if (diag) launch_dep(lbm_batch_kernel<float, true, 0, TY, FEW>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<float, false, 0, TY, FEW>, ctas, block, 0, s, b);
   }
+}
+
+cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, bool columns,
+                             cudaStream_t s) {
+  if (columns) launch_batch_few<false>(b, diag, all, s);
+  else launch_batch_few<true>(b, diag, all, s);
   return cudaGetLastError();
 }
 

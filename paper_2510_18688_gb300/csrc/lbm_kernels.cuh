@@ -57,6 +57,16 @@ struct Shape {
   static constexpr int TY = TY_, HY = TY_ + 2, HN = HX * HY, NT = TX * TY_, RING = HN - NT;
 };
 __host__ __device__ constexpr int tiles_y(int ny, int ty) { return (ny + ty - 1) / ty; }
+// One-dimensional columns: fewer than 32 rows, at least four times as long,
+// at most 32768 nodes.  They stay with the fused tile from global loads.  In
+// double the node step is the faster one there too (512 x 8: 14.6 us a step;
+// fused 57 us on 32 x 8 tiles, 42 us on 32 x 1), in float the TMA-staged tile
+// takes as long (9 us, latency alone); but across a column the velocity is
+// nothing but rounding (1e-20 against 4e-5 along it), and the fused tile keeps
+// every bit of it as earlier results and saved runs have it.
+__host__ __device__ inline bool is_column(int nx, int ny) {
+  return ny < 32 && nx >= 4 * ny && (long long)nx * ny <= 32768;
+}
 enum { BC_PERIODIC = 0, BC_DIRICHLET = 1, BC_ADIABATIC = 2 };
 enum { LAT_FLOW = 1, LAT_PHASE = 2, LAT_HEAT = 4 };
 enum { LAG_FL = 0, LAG_W, LAG_P, LAG_PHUX, LAG_PHUY, LAG_Q, NLAG };

@@ -20,16 +20,10 @@ inline dim3 grid_dims(const Geom& g, int ty = TY) {
 // on 32 x ty tiles (ty = 4, 8 or 16), MODE_READ on 32 x 8.
 cudaError_t launch_step_f32(const Args<float>& a, int mode, bool diag, cudaStream_t s,
                             int ty = TY);
-// Double on grids of fewer than THIN_ROWS rows and at most THIN_NODES nodes
-// -- the one-dimensional columns -- stays with the fused tile: MODE_STEP on
-// 32 x ty tiles (ty = 1, 2 or 4), MODE_READ and batches on 32 x THIN_TY.  The
-// node step is the faster one there too (512 x 8: 14.6 us a step; fused 57 us
-// on 32 x 8 tiles, 42 us on 32 x 1), but across a column the velocity is
-// nothing but rounding (1e-20 against 4e-5 along it), and the fused tile
-// keeps every bit of it as earlier results and saved runs have it.  One warp
-// a tile spreads a column over the most SMs; with it the step is a single
-// warp's chain of FP64 latencies whatever the size up to the bound.
-constexpr int THIN_ROWS = 32, THIN_NODES = 32768, THIN_TY = 1;
+// Double columns: MODE_STEP on 32 x ty tiles (ty = 1, 2 or 4), MODE_READ and
+// batches on 32 x THIN_TY.  One warp a tile spreads a column over the most
+// SMs; a step is then a single warp's chain of FP64 latencies at any size.
+constexpr int THIN_TY = 1;
 cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s, int ty);
 cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s);
 // The diagnostics of a caller-held double state, which has no room for the
@@ -63,7 +57,9 @@ cudaError_t launch_adjoint_reduce(const double* acc, const Geom& g, double* out,
 // Forward-mode tangent (FP64 value and derivative).
 cudaError_t launch_init_tan(const InitArgs<Dual>& a, cudaStream_t s);
 // Up to BATCH_MAX_GRIDS grids in one launch, one CTA per tile.
-cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, cudaStream_t s);
+// (all columns, or none)
+cudaError_t launch_batch_f32(const BatchTable<float>& b, bool diag, bool all, bool columns,
+                             cudaStream_t s);
 // Grid-wide diagnostics from the partial sums (one CTA per diagnostic).
 cudaError_t launch_diag_finalize(const double* partial, int nb, double* out, long long step,
                                  cudaStream_t s);

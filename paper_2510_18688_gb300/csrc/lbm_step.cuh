@@ -12,6 +12,7 @@
 #pragma once
 
 #include "lbm_kernels.cuh"
+#include "lbm_wb.cuh"
 
 // resident CTAs per SM the float kernel is compiled for (register budget)
 #ifndef LBM_MIN_BLOCKS_F32
@@ -510,9 +511,9 @@ __device__ __forceinline__ void node_macros(const Geom& g, const Coef<R>& c, int
 // The node's contributions to the FP64 diagnostics (lbm_diag order) and a
 // non-finite flag: a non-finite population anywhere makes one of the sums
 // non-finite.
-template <typename R>
+template <typename R, typename MT>
 __device__ __forceinline__ void diag_values(const Coef<R>& c, int lat, const Local<R>& L,
-                                            const Macro<R>& M, R sg, R sh, const R* f,
+                                            const MT& M, R sg, R sh, const R* f,
                                             R* dvals) {
   dvals[0] = L.rho;
   dvals[1] = L.w * (c.rho_s * (R(1) - L.fl) + c.rho_l * L.fl);
@@ -534,8 +535,10 @@ __device__ __forceinline__ void diag_values(const Coef<R>& c, int lat, const Loc
 // TX x TYS nodes (a Shape).  b / nb: the tile's index and the grid's tile
 // count for the diagnostic partials (b < 0: taken from the CTA's position in
 // its grid).  LATC: compile-time lattice set (7 = all three) or 0 (read at
-// run time).  Every thread of the CTA calls it.
-template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY>
+// run time).  FEW: a float step's phase B in the form of lbm_wb.cuh.  Every
+// thread of the CTA calls it.
+template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY,
+          bool FEW = false>
 __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, int b, int nb) {
   // the tile's shape; these hide the namespace's 32 x 8 constants
   constexpr int TY = Shape<TYS>::TY, HN = Shape<TYS>::HN, NT = Shape<TYS>::NT;
@@ -699,7 +702,8 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
   {
     const int hi = (ty + 1) * HX + (tx + 1);
     s_phi[hi] = L.phi;
-    s_fs[hi] = L.fs;
+    if constexpr (FEW) s_fs[hi] = fmaf(c.cos_th, phi0, c.cos_ps * L.fs);
+    else s_fs[hi] = L.fs;
     s_rho[hi] = L.rho;
     s_p[hi] = pp;
     s_phi0[hi] = phi0;
@@ -739,7 +743,8 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     if constexpr (WB) Lq = local_state_wb(c, lat, sgq, shq, s_rfl[k], wq, s_rQ[k], Tq, Cq, q0);
     else Lq = local_state(c, lat, sgq, shq, s_rfl[k], wq, s_rQ[k], q0);
     s_phi[hi] = Lq.phi;
-    s_fs[hi] = Lq.fs;
+    if constexpr (FEW) s_fs[hi] = fmaf(c.cos_th, q0, c.cos_ps * Lq.fs);
+    else s_fs[hi] = Lq.fs;
     s_rho[hi] = Lq.rho;
     if constexpr (WB) s_T[hi] = Lq.T;
   };
@@ -755,8 +760,72 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
   // Instantiated twice: for a tile whose nodes and ring are all inside the
   // grid (block-uniform branch) every node is valid and every link stays in
   // the grid, so that path carries no boundary logic at all.
+  auto phase_b_few = [&](auto interior) {
+   if constexpr (FEW) {
+    constexpr bool IN = decltype(interior)::value;
+    R dvals[NDIAG];
+    MacroWb M;
+    const Links<IN> k(g, gx, gy);
+    const bool valid_n = IN || valid;
+    const int hc = (ty + 1) * HX + (tx + 1);
+    if (valid_n) {
+      M = macros_wb<IN>(c, lat, k, L, phi0, f, s_phi + hc, s_fs + hc, s_rho + hc, s_p + hc, HX);
+      if (DIAG) diag_values(c, lat, L, M, sg, sh, f, dvals);
+    } else if (DIAG) {
+#pragma unroll
+      for (int q = 0; q < NDIAG; q++) dvals[q] = R(0);
+    }
+    if (DIAG) block_diag_warps(dvals, s_red, tid);
+    if (!valid_n) return;
+    S* out = a.pout;
+    const R Tq = (lat & LAT_HEAT) ? s_Tp[0][tid] : R(0), Cq = (lat & LAT_HEAT) ? s_Tp[WB ? 1 : 0][tid] : R(0);
+    const R CT = cap_rn(c, L.fs, L.w) * L.T;
+    if (lat & LAT_FLOW) flow_wb<IN>(c, out, P, n, k, f, L.rho, M);
+    if (lat & LAT_PHASE) {
+      R gq[9];
+#pragma unroll
+      for (int i = 0; i < 9; i++) gq[i] = STASH ? s_pop[i][tid] : ldp(pn + (9 + i) * P);
+      if (STASH) {
+        phuxp = s_phu[0][tid];
+        phuyp = s_phu[STASH ? 1 : 0][tid];
+      }
+      const R dref = ref_delta(rest_ref_g(L.w, phi0), rest_ref_g(wp, phi0));
+      phase_wb<IN>(c, out + 9 * P, P, n, k, gq, L.phi, L.phir, L.mdot, phuxp, phuyp, M, dref);
+    }
+    if (lat & LAT_HEAT) {
+      R hq[9];
+      if (STASH) {
+#pragma unroll
+        for (int i = 0; i < 9; i++) hq[i] = s_pop[STASH ? 9 + i : 0][tid];
+      } else if (masked) {
+        cold_mask_h(c, wp, phi0, hq);
+        hq[0] -= ref_h0(c, wp, flp, Tq, Cq);
+#pragma unroll
+        for (int i = 1; i < 9; i++) hq[i] -= ref_hi(i <= 4 ? c.wrr1 : c.wrr5, Tq);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 9; i++) hq[i] = ldp(pn + (18 + i) * P);
+      }
+      const R dref0 = ref_delta(ref_h0(c, L.w, L.fl, L.T, cap_rn(c, L.fs, L.w)),
+                                ref_h0(c, wp, flp, Tq, Cq));
+      heat_wb<IN>(g, c, out + 18 * P, P, n, k, hq, L, CT, L.T - Tq, L.rhoHr, M,
+                  ref_hi(c.wrr1, Tq), ref_hi(c.wrr5, Tq), dref0, s_T + hc);
+    }
+    a.lout[LAG_FL * P + n] = L.fl;
+    a.lout[LAG_W * P + n] = L.w;
+    a.lout[LAG_P * P + n] = (lat & LAT_FLOW) ? M.pr : R(0);
+    a.lout[LAG_PHUX * P + n] = (lat & LAT_PHASE) ? M.phux : R(0);
+    a.lout[LAG_PHUY * P + n] = (lat & LAT_PHASE) ? M.phuy : R(0);
+    a.lout[LAG_Q * P + n] = (lat & LAT_HEAT) ? CT * L.mdot : R(0);
+    a.lout[LAG_T * P + n] = L.T;
+   }
+  };
   auto phase_b = [&](auto interior) {
   constexpr bool IN = decltype(interior)::value;
+  if constexpr (FEW) {
+    phase_b_few(interior);
+    return;
+  } else {
   R dvals[NDIAG];
   Macro<R> M;
   // links that stay inside the grid need no boundary logic
@@ -862,6 +931,7 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
         if (a.out[k]) put_out(a.out[k], d, (long long)g.nx * g.ny, vals[k]);
     }
   }
+  }
   };
   // short tiles take the path of the 32 x 8 tile they are part of: the two
   // copies of the arithmetic may round differently, so a node's last bits do
@@ -880,12 +950,13 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
 
 // One CTA per 32 x TYS tile; float kernels keep the 64-register budget of
 // the 32 x 8 shape (4 CTAs of 256 threads per SM) at every shape.
-template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY>
+template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY,
+          bool FEW = false>
 __global__ void __launch_bounds__(Shape<TYS>::NT,
                                   sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 * TY / TYS : 1)
     lbm_step_kernel(const Args<R, S> a) {
   after_previous();
-  step_tile<R, MODE, DIAG, LATC, S, TYS>(a, blockIdx.x, blockIdx.y, -1, 0);
+  step_tile<R, MODE, DIAG, LATC, S, TYS, FEW>(a, blockIdx.x, blockIdx.y, -1, 0);
 }
 
 // Many independent grids (uneven sizes and parameters) advanced in one
@@ -904,7 +975,7 @@ struct BatchTable {
   Args<R> args[BATCH_MAX_GRIDS];
 };
 
-template <typename R, bool DIAG, int LATC, int TYS = TY>
+template <typename R, bool DIAG, int LATC, int TYS = TY, bool FEW = false>
 __global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
     lbm_batch_kernel(const __grid_constant__ BatchTable<R> B) {
   after_previous();
@@ -919,7 +990,8 @@ __global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCK
   const int local = t - B.tile_base[lo];
   const int tiles_x = (a.g.nx + TX - 1) / TX;
   const int ntiles = B.tile_base[lo + 1] - B.tile_base[lo];
-  step_tile<R, MODE_STEP, DIAG, LATC, R, TYS>(a, local % tiles_x, local / tiles_x, local, ntiles);
+  step_tile<R, MODE_STEP, DIAG, LATC, R, TYS, FEW>(a, local % tiles_x, local / tiles_x, local,
+                                                   ntiles);
 }
 
 }  // namespace lbmk

@@ -27,8 +27,8 @@
 // sets *status and the CTA drains its copies and leaves.
 #pragma once
 
-#include "lbm_step.cuh"
 #include "lbm_tma.cuh"
+#include "lbm_wb.cuh"
 
 namespace lbmk {
 
@@ -89,6 +89,12 @@ constexpr size_t tile_smem_bytes(int nst) {
 template <int NST>
 constexpr int tile_min_blocks() {
   return NST == 2 ? 2 : 3;
+}
+
+// the status word is host memory the device writes
+__device__ __forceinline__ void report_timeout(unsigned* status) {
+  *(volatile unsigned*)status = 1u;
+  __threadfence_system();
 }
 
 __device__ __forceinline__ float lds(const float* p) { return *p; }
@@ -171,7 +177,7 @@ __device__ __forceinline__ TileMask tile_mask(const Args<float, S>& a, int x0, i
 template <typename S, bool DIAG, int LATC>
 __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileStage<S>& st,
                                           int bx, int by, int b, int nb, float* s_phi,
-                                          float* s_fs, float* s_rho, float* s_T,
+                                          float* s_wet, float* s_rho, float* s_T,
                                           float (*s_red)[NDIAG], TileMask mk) {
   using St = TileStage<S>;
   using R = float;
@@ -196,7 +202,7 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
   // ---- phase A1: own node -------------------------------------------------
   const R phi0 = st.phi0[ty + 1][tx + St::XL];
   const R flp = lag[LAG_FL * PL + cl], wp = lag[LAG_W * PL + cl];
-  const R pp = lag[LAG_P * PL + cl], Qp = lag[LAG_Q * PL + cl];
+  const R Qp = lag[LAG_Q * PL + cl];
   const bool masked = (lat & LAT_HEAT) && mk.own;
   R Tp = R(0), Cp = R(0);
   if (lat & LAT_HEAT) {
@@ -225,9 +231,25 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
   }
   const Local<R> L = local_state_wb(c, lat, sg, sh, flp, wp, Qp, Tp, Cp, phi0);
   s_phi[hc] = L.phi;
-  s_fs[hc] = L.fs;
+  s_wet[hc] = fmaf(c.cos_th, phi0, c.cos_ps * L.fs);
   s_rho[hc] = L.rho;
   s_T[hc] = L.T;
+  // What depends on the local state alone is finished here -- the new heat
+  // capacity, the changes of the rest references, most lags -- so that little
+  // stays in registers through phase B: at 64 registers every spilled value
+  // goes to L2, with the L1 storage carved out as shared memory.
+  const R cap = cap_rn(c, L.fs, L.w);
+  const R CT = cap * L.T;
+  const R dref_g = ref_delta(rest_ref_g(L.w, phi0), rest_ref_g(wp, phi0));
+  R dref_h = R(0);
+  if (lat & LAT_HEAT)
+    dref_h = ref_delta(ref_h0(c, L.w, L.fl, L.T, cap), ref_h0(c, wp, flp, Tp, Cp));
+  if (valid) {
+    a.lout[LAG_FL * P + n] = L.fl;
+    a.lout[LAG_W * P + n] = L.w;
+    a.lout[LAG_Q * P + n] = (lat & LAT_HEAT) ? CT * L.mdot : R(0);
+    a.lout[LAG_T * P + n] = L.T;
+  }
 
   // ---- phase A2: the ring ----------------------------------------------------
   if (tid < RING) {
@@ -265,7 +287,7 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
     }
     const Local<R> Lq = local_state_wb(c, lat, sgq, shq, flq, wq, Qq, Tq, Cq, q0);
     s_phi[hi] = Lq.phi;
-    s_fs[hi] = Lq.fs;
+    s_wet[hi] = fmaf(c.cos_th, q0, c.cos_ps * Lq.fs);
     s_rho[hi] = Lq.rho;
     s_T[hi] = Lq.T;
   }
@@ -278,8 +300,8 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
   auto phase_b = [&](auto interior) {
   constexpr bool IN = decltype(interior)::value;
   R dvals[NDIAG];
-  Macro<R> M;
-  const bool inner = IN || (gx > 0 && gx < g.nx - 1 && gy > 0 && gy < g.ny - 1);
+  MacroWb M;
+  const Links<IN> k(g, gx, gy);
   const bool valid_n = IN || valid;
   R f[9];
   if (valid_n) {
@@ -287,62 +309,45 @@ __device__ __forceinline__ void tile_step(const Args<float, S>& a, const TileSta
 #pragma unroll
       for (int i = 0; i < 9; i++) f[i] = lds(&st.f[i][ty][tx]);
     }
-    node_macros<R, true>(g, c, lat, gx, gy, inner, L, phi0, pp, f, s_phi + hc, s_fs + hc,
-                         s_rho + hc, HX, lag + LAG_P * PL + cl, &st.phi0[ty + 1][tx + St::XL],
-                         St::WL, M);
+    M = macros_wb<IN>(c, lat, k, L, st.phi0[ty + 1][tx + St::XL], f, s_phi + hc, s_wet + hc,
+                      s_rho + hc, lag + LAG_P * PL + cl, St::WL);
+    a.lout[LAG_P * P + n] = (lat & LAT_FLOW) ? M.pr : R(0);
+    a.lout[LAG_PHUX * P + n] = (lat & LAT_PHASE) ? M.phux : R(0);
+    a.lout[LAG_PHUY * P + n] = (lat & LAT_PHASE) ? M.phuy : R(0);
     if (DIAG) diag_values(c, lat, L, M, sg, sh, f, dvals);
   } else if (DIAG) {
 #pragma unroll
-    for (int k = 0; k < NDIAG; k++) dvals[k] = R(0);
+    for (int q = 0; q < NDIAG; q++) dvals[q] = R(0);
   }
   if (DIAG) block_diag_warps(dvals, s_red, tid);
 
   if (valid_n) {
     S* out = a.pout;
-    if (lat & LAT_FLOW) {
-      if (inner) collide_flow_wb<true>(g, c, out, P, gx, gy, n, f, L.rho, M);
-      else collide_flow_wb<false>(g, c, out, P, gx, gy, n, f, L.rho, M);
-    }
+    if (lat & LAT_FLOW) flow_wb<IN>(c, out, P, n, k, f, L.rho, M);
     if (lat & LAT_PHASE) {
       R gq[9];
 #pragma unroll
       for (int i = 0; i < 9; i++) gq[i] = lds(gh + i * PG + cg);
       const R phuxp = lag[LAG_PHUX * PL + cl], phuyp = lag[LAG_PHUY * PL + cl];
-      const R dref = ref_delta(rest_ref_g(L.w, phi0), rest_ref_g(wp, phi0));
-      if (inner)
-        collide_phase<R, true>(g, c, out + 9 * P, P, gx, gy, n, gq, L.phi, L.phir, L.mdot,
-                               phuxp, phuyp, M, dref);
-      else
-        collide_phase<R, false>(g, c, out + 9 * P, P, gx, gy, n, gq, L.phi, L.phir, L.mdot,
-                                phuxp, phuyp, M, dref);
+      phase_wb<IN>(c, out + 9 * P, P, n, k, gq, L.phi, L.phir, L.mdot, phuxp, phuyp, M, dref_g);
     }
     if (lat & LAT_HEAT) {
       R hq[9];
+      const R Tq = lag[LAG_T * PL + cl];
       if (masked) {
-        cold_mask_h(c, wp, phi0, hq);
-        hq[0] -= ref_h0(c, wp, flp, Tp, Cp);
+        const R wq = lag[LAG_W * PL + cl], fq = lag[LAG_FL * PL + cl];
+        const R q0 = st.phi0[ty + 1][tx + St::XL];
+        cold_mask_h(c, wq, q0, hq);
+        hq[0] -= ref_h0(c, wq, fq, Tq, cap_rn(c, fs_rn(wq, fq, q0), wq));
 #pragma unroll
-        for (int i = 1; i < 9; i++) hq[i] -= ref_hi(i <= 4 ? c.wrr1 : c.wrr5, Tp);
+        for (int i = 1; i < 9; i++) hq[i] -= ref_hi(i <= 4 ? c.wrr1 : c.wrr5, Tq);
       } else {
 #pragma unroll
         for (int i = 0; i < 9; i++) hq[i] = lds(gh + (9 + i) * PG + cg);
       }
-      const R dref0 = ref_delta(ref_h0(c, L.w, L.fl, L.T, M.cap), ref_h0(c, wp, flp, Tp, Cp));
-      const R aold = ref_hi(c.wrr1, Tp), dold = ref_hi(c.wrr5, Tp);
-      if (inner)
-        collide_heat_wb<true>(g, c, out + 18 * P, P, gx, gy, n, hq, L.fs, L.w, L.T, L.T - Tp,
-                              L.rhoHr, L.mdot, M, aold, dold, dref0, s_T, hc);
-      else
-        collide_heat_wb<false>(g, c, out + 18 * P, P, gx, gy, n, hq, L.fs, L.w, L.T, L.T - Tp,
-                               L.rhoHr, L.mdot, M, aold, dold, dref0, s_T, hc);
+      heat_wb<IN>(g, c, out + 18 * P, P, n, k, hq, L, CT, L.T - Tq, L.rhoHr, M,
+                  ref_hi(c.wrr1, Tq), ref_hi(c.wrr5, Tq), dref_h, s_T + hc);
     }
-    a.lout[LAG_FL * P + n] = L.fl;
-    a.lout[LAG_W * P + n] = L.w;
-    a.lout[LAG_P * P + n] = (lat & LAT_FLOW) ? M.pr : R(0);
-    a.lout[LAG_PHUX * P + n] = (lat & LAT_PHASE) ? M.phux : R(0);
-    a.lout[LAG_PHUY * P + n] = (lat & LAT_PHASE) ? M.phuy : R(0);
-    a.lout[LAG_Q * P + n] = (lat & LAT_HEAT) ? M.cap * L.T * L.mdot : R(0);
-    a.lout[LAG_T * P + n] = L.T;
   }
   };
   if (x0 >= 1 && x0 + TX < g.nx && y0 >= 1 && y0 + TY < g.ny) phase_b(std::true_type{});
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(NT, tile_min_blocks<NST>())
   extern __shared__ unsigned char tile_smem[];
   St* stage = reinterpret_cast<St*>(tile_smem + ((128u - (smem_u32(tile_smem) & 127u)) & 127u));
   __shared__ __align__(8) uint64_t bar[NST];
-  __shared__ float s_phi[HN], s_fs[HN], s_rho[HN], s_T[HN];
+  __shared__ float s_phi[HN], s_wet[HN], s_rho[HN], s_T[HN];
   __shared__ float s_red[NT / 32][NDIAG];
   const int tid = threadIdx.y * TX + threadIdx.x;
   if (tid == 0) {
@@ -392,7 +397,7 @@ __global__ void __launch_bounds__(NT, tile_min_blocks<NST>())
     }
     tile_fix_edges(ta.a, stage[s], bx * TX, by * TY, tid);
     __syncthreads();
-    tile_step<S, DIAG, LATC>(ta.a, stage[s], bx, by, t, ta.ntiles, s_phi, s_fs, s_rho, s_T,
+    tile_step<S, DIAG, LATC>(ta.a, stage[s], bx, by, t, ta.ntiles, s_phi, s_wet, s_rho, s_T,
                              s_red, mk);
     // this thread's reads (and edge writes) of stage s come before the TMA
     // writes that will refill it
@@ -402,7 +407,7 @@ __global__ void __launch_bounds__(NT, tile_min_blocks<NST>())
     if (NST == 1 && tid == 0 && tn < ta.ntiles) tile_issue(ta, stage[0], &bar[0], tn);
   }
   if (timed_out && tid == 0) {
-    atomicExch(ta.status, 1u);
+    report_timeout(ta.status);
     // drain: the late copy and (two stages) the prefetch of the next tile,
     // if issued, must land before the CTA's shared memory goes away
     if (NST == 2) {
@@ -429,7 +434,7 @@ __device__ __forceinline__ void tile_once(const Args<float, S>& a, const CUtenso
   extern __shared__ unsigned char tile_smem[];
   St* stage = reinterpret_cast<St*>(tile_smem + ((128u - (smem_u32(tile_smem) & 127u)) & 127u));
   __shared__ __align__(8) uint64_t bar;
-  __shared__ float s_phi[HN], s_fs[HN], s_rho[HN], s_T[HN];
+  __shared__ float s_phi[HN], s_wet[HN], s_rho[HN], s_T[HN];
   __shared__ float s_red[NT / 32][NDIAG];
   const int tid = threadIdx.y * TX + threadIdx.x;
   if (tid == 0) {
@@ -445,14 +450,14 @@ __device__ __forceinline__ void tile_once(const Args<float, S>& a, const CUtenso
   const bool ok = mbar_wait(&bar, 0);
   if (__syncthreads_or(!ok)) {
     if (tid == 0) {
-      atomicExch(status, 1u);
+      report_timeout(status);
       mbar_wait(&bar, 0);  // the late copy must land before the CTA leaves
     }
     return;
   }
   tile_fix_edges(a, stage[0], bx * TX, by * TY, tid);
   __syncthreads();
-  tile_step<S, DIAG, LATC>(a, stage[0], bx, by, b, nb, s_phi, s_fs, s_rho, s_T, s_red, mk);
+  tile_step<S, DIAG, LATC>(a, stage[0], bx, by, b, nb, s_phi, s_wet, s_rho, s_T, s_red, mk);
 }
 
 // CTAs per SM of the loop-free one-stage kernels: four for one grid (64

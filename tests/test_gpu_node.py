@@ -1,5 +1,5 @@
 """The double-precision node step: grids at the edges of its warps, blocks and
-of the rule that leaves grids of few rows to the fused tile; batches that mix
+of the rule that leaves one-dimensional columns to the fused tile; batches that mix
 the two; the reciprocal its kernels take."""
 from fractions import Fraction
 
@@ -29,8 +29,8 @@ def _close(got, ref, tol=1e-10):  # the parity bar of the FP64 step
         assert np.abs(got[k] - ref[k]).max() <= tol * scale + 1e-18, k
 
 
-# columns of one warp and less, rows that end inside a warp and a block, one
-# row to each side of the rule's 32 rows, and of its 32768 nodes
+# columns of one warp and less, rows that end inside a warp and a block, and
+# both sides of the rule for one-dimensional columns
 SIZES = [(2, 32), (3, 33), (31, 32), (32, 32), (33, 32), (33, 31), (64, 64), (129, 33), (40, 200),
          (1057, 31), (1060, 31), (701, 39)]
 
@@ -53,7 +53,7 @@ def test_sizes_match_the_oracle(env, nx, ny, seed):
     s.close()
 
 
-# (grids of fewer rows take the fused tile, whose copies with and without sums
+# (columns take the fused tile, whose copies with and without sums
 # round some nodes differently)
 @pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny", [z for z in SIZES if z[1] >= 32])
