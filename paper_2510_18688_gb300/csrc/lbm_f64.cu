@@ -1,25 +1,33 @@
 // lbm_f64.cu -- double-precision kernels beside the node step (sm_103a): the
 // initial state, the diagnostics of a caller-held state, crossings, and the
 // sum of the diagnostic partials.
+#include "lbm_column.cuh"
 #include "lbm_launch.h"
 
 namespace lbmk {
 
 template <int MODE, bool DIAG, int TYS>
 static void launch_one(const Args<double>& a, cudaStream_t s) {
-  const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS);
+  constexpr int RW = TYS == THIN_TY ? THIN_RING_WARPS : 0;
+  const dim3 grid = grid_dims(a.g, TYS), block = block_dims(TYS + RW);
   // the all-lattices case is specialised at compile time
   if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
-    launch_dep(lbm_step_kernel<double, MODE, DIAG, 7, double, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<double, MODE, DIAG, 7, double, TYS, false, RW>, grid, block, 0, s, a);
   else
-    launch_dep(lbm_step_kernel<double, MODE, DIAG, 0, double, TYS>, grid, block, 0, s, a);
+    launch_dep(lbm_step_kernel<double, MODE, DIAG, 0, double, TYS, false, RW>, grid, block, 0, s, a);
 }
 
+// Columns: steps without sums on four warps a tile; steps with sums, whose
+// compiled order of rounding differs from theirs, as step_tile's.
 template <bool DIAG>
 static void launch_shape(const Args<double>& a, int ty, cudaStream_t s) {
-  if (ty == 1) launch_one<MODE_STEP, DIAG, 1>(a, s);
-  else if (ty == 2) launch_one<MODE_STEP, DIAG, 2>(a, s);
-  else launch_one<MODE_STEP, DIAG, 4>(a, s);
+  if (ty == 2) launch_one<MODE_STEP, DIAG, 2>(a, s);
+  else if (ty == 4) launch_one<MODE_STEP, DIAG, 4>(a, s);
+  else if (DIAG) launch_one<MODE_STEP, true, THIN_TY>(a, s);
+  else if (a.g.lattices == (LAT_FLOW | LAT_PHASE | LAT_HEAT))
+    launch_dep(lbm_column_kernel<7>, grid_dims(a.g, THIN_TY), column_dims(), 0, s, a);
+  else
+    launch_dep(lbm_column_kernel<0>, grid_dims(a.g, THIN_TY), column_dims(), 0, s, a);
 }
 
 cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s, int ty) {
@@ -34,14 +42,16 @@ cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStre
 }
 
 cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s) {
-  const dim3 block = block_dims(THIN_TY);
+  constexpr int RW = THIN_RING_WARPS;
+  const dim3 block = block_dims(THIN_TY + RW);
   const int ctas = b.tile_base[b.ngrids];
-  if (all) {
-    if (diag) launch_dep(lbm_batch_kernel<double, true, 7, THIN_TY>, ctas, block, 0, s, b);
-    else launch_dep(lbm_batch_kernel<double, false, 7, THIN_TY>, ctas, block, 0, s, b);
+  if (diag) {
+    if (all)
+      launch_dep(lbm_batch_kernel<double, true, 7, THIN_TY, false, RW>, ctas, block, 0, s, b);
+    else launch_dep(lbm_batch_kernel<double, true, 0, THIN_TY, false, RW>, ctas, block, 0, s, b);
   } else {
-    if (diag) launch_dep(lbm_batch_kernel<double, true, 0, THIN_TY>, ctas, block, 0, s, b);
-    else launch_dep(lbm_batch_kernel<double, false, 0, THIN_TY>, ctas, block, 0, s, b);
+    if (all) launch_dep(lbm_column_batch_kernel<7>, ctas, column_dims(), 0, s, b);
+    else launch_dep(lbm_column_batch_kernel<0>, ctas, column_dims(), 0, s, b);
   }
   return cudaGetLastError();
 }

@@ -60,7 +60,7 @@ __host__ __device__ constexpr int tiles_y(int ny, int ty) { return (ny + ty - 1)
 // One-dimensional columns: fewer than 32 rows, at least four times as long,
 // at most 32768 nodes.  They stay with the fused tile from global loads.  In
 // double the node step is the faster one there too (512 x 8: 14.6 us a step;
-// fused 57 us on 32 x 8 tiles, 42 us on 32 x 1), in float the TMA-staged tile
+// fused 57 us on 32 x 8 tiles, 19 us on 32 x 1 with four warps), in float the TMA-staged tile
 // takes as long (9 us, latency alone); but across a column the velocity is
 // nothing but rounding (1e-20 against 4e-5 along it), and the fused tile keeps
 // every bit of it as earlier results and saved runs have it.
@@ -485,12 +485,25 @@ __device__ __forceinline__ Local<float> local_state_wb(const Coef<float>& c, int
 }
 
 // Eq. (6) without the Laplacian terms.
-template <typename R>
+// a b + c d.  Which product of such a sum the compiler rounds before the FMA
+// is its own choice and changes with the code around it.  PIN = 1 rounds c d,
+// PIN = 2 rounds a b: a kernel that has to give the bits of an earlier one
+// states the order (lbm_column.cuh).
+template <int PIN, typename R>
+__device__ __forceinline__ R sum2(R a, R b, R c, R d) {
+  if constexpr (PIN == 1) return fma(a, b, c * d);
+  else if constexpr (PIN == 2) return fma(c, d, a * b);
+  else return a * b + c * d;
+}
+
+template <typename R, bool PIN = false>
 __device__ __forceinline__ R chem_local(const Coef<R>& c, R phi, R phi0, R fs) {
+  constexpr int P1 = PIN ? 1 : 0, P2 = PIN ? 2 : 0;
   const R s3 = c.s3, s9 = c.s9;
-  return s3 * phi * (phi - R(1)) * (phi + R(1)) + s9 * phi0 * phi0 * phi +
-         s3 * c.cos_th * phi0 * (R(3) * phi * phi + phi0 * phi0 - R(1)) + s9 * fs * fs * phi +
-         s3 * c.cos_ps * fs * (R(3) * phi * phi + fs * fs - R(1));
+  return sum2<P1, R>(s3 * phi * (phi - R(1)), phi + R(1), s9 * phi0 * phi0, phi) +
+         s3 * c.cos_th * phi0 * (sum2<P2, R>(R(3) * phi, phi, phi0, phi0) - R(1)) +
+         s9 * fs * fs * phi +
+         s3 * c.cos_ps * fs * (sum2<P2, R>(R(3) * phi, phi, fs, fs) - R(1));
 }
 
 __device__ __forceinline__ int wrap_or_clamp(int v, int n, int bc_lo, int bc_hi) {

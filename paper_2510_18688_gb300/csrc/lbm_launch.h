@@ -24,6 +24,7 @@ cudaError_t launch_step_f32(const Args<float>& a, int mode, bool diag, cudaStrea
 // batches on 32 x THIN_TY.  One warp a tile spreads a column over the most
 // SMs; a step is then a single warp's chain of FP64 latencies at any size.
 constexpr int THIN_TY = 1;
+constexpr int THIN_RING_WARPS = 3;  // for the tile's ring of 70 nodes
 cudaError_t launch_step_f64(const Args<double>& a, int mode, bool diag, cudaStream_t s, int ty);
 cudaError_t launch_batch_f64(const BatchTable<double>& b, bool diag, bool all, cudaStream_t s);
 // The diagnostics of a caller-held double state, which has no room for the

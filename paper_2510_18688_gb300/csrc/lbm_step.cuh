@@ -82,11 +82,13 @@ struct Macro {
 // each pair costs one evaluation of each part.  Pairs: (1,3), (2,4) with
 // weight 1/9 and (5,7), (6,8) with weight 1/36.
 
-// Flow collision Eqs. (11), (14)-(16) and push.
-template <typename R, bool INNER, typename S>
+// Flow collision Eqs. (11), (14)-(16) and push.  PIN: the rest population's
+// sums of products contracted in a stated order (sum2); in_tile: the order of
+// step_tile's copy for tiles inside the grid, else of its other copy.
+template <typename R, bool INNER, bool PIN = false, typename S>
 __device__ __forceinline__ void collide_flow(const Geom& g, const Coef<R>& c, S* __restrict__ out,
                                              int P, int x, int y, int n, const R* f, R rho,
-                                             const Macro<R>& M) {
+                                             const Macro<R>& M, bool in_tile = false) {
   const R itau = qdiv(R(1), M.tauf);
   const R omi = R(1) - itau;
   const R fcoef = R(1) - R(0.5) * itau;
@@ -98,9 +100,15 @@ __device__ __forceinline__ void collide_flow(const Geom& g, const Coef<R>& c, S*
   {
     R F0 = fsym0;
     if (iso) F0 += M.S * (R(0) - R(2) / R(3)) * R(1.5);
-    const R feq0 = M.pr * R(3) * (qw<R>(0) - R(1)) + rho * qw<R>(0) * (-R(1.5) * M.uu);
-    push<R, INNER, false>(g, c, out, P, 0, x, y, n,
-                          f[0] * omi + itau * feq0 + fcoef * qw<R>(0) * F0);
+    const R feq0 =
+        sum2<PIN ? 2 : 0, R>(M.pr * R(3), qw<R>(0) - R(1), rho * qw<R>(0), -R(1.5) * M.uu);
+    if constexpr (PIN) {
+      const R rest = in_tile ? sum2<1, R>(f[0], omi, itau, feq0) : sum2<2, R>(f[0], omi, itau, feq0);
+      push<R, INNER, false>(g, c, out, P, 0, x, y, n, fma(fcoef * qw<R>(0), iso ? F0 : fma(-R(3), M.uFt, M.S), rest));
+    } else {
+      push<R, INNER, false>(g, c, out, P, 0, x, y, n,
+                            f[0] * omi + itau * feq0 + fcoef * qw<R>(0) * F0);
+    }
   }
 #pragma unroll
   for (int i = 1; i <= 8; i++) {
@@ -349,20 +357,21 @@ __device__ __forceinline__ void collide_heat_wb(const Geom& g, const Coef<float>
 // gradient of a large field (the pressure of a compressed gas, ~1e-9 per node
 // against p ~ 6e-4) keeps its relative precision instead of being lost in
 // the rounding of the products w_i v.
-template <typename R>
+template <typename R, bool PIN = false>
 __device__ __forceinline__ void grad_pairs(const R* v, int s, R& gx, R& gy) {
   const R d13 = v[1] - v[-1], d24 = v[s] - v[-s];
   const R d57 = v[s + 1] - v[-s - 1], d86 = v[-s + 1] - v[s - 1];
-  gx = qw<R>(1) * d13 + qw<R>(5) * (d57 + d86);
-  gy = qw<R>(1) * d24 + qw<R>(5) * (d57 - d86);
+  gx = sum2<PIN ? 1 : 0, R>(qw<R>(1), d13, qw<R>(5), d57 + d86);
+  gy = sum2<PIN ? 1 : 0, R>(qw<R>(1), d24, qw<R>(5), d57 - d86);
 }
 
-template <typename R, bool WB>
+template <typename R, bool WB, bool PIN = false>
 __device__ __forceinline__ void node_macros(const Geom& g, const Coef<R>& c, int lat, int gx,
                                             int gy, bool inner, const Local<R>& L, R phi0, R pp,
                                             R* f, const R* cphi, const R* cfs,
                                             const R* crho, int sh, const R* cp,
                                             const R* cphi0, int sb, Macro<R>& M) {
+  constexpr int P1 = PIN ? 1 : 0;
   R gphx = R(0), gphy = R(0), lphi = R(0), lphi0 = R(0), lfs = R(0);
   R grx = R(0), gry = R(0), gpx = R(0), gpy = R(0);
   if (lat & LAT_PHASE) {
@@ -377,11 +386,16 @@ __device__ __forceinline__ void node_macros(const Geom& g, const Coef<R>& c, int
     grad_pairs(cphi, sh, gphx, gphy);
   }
   if (lat & LAT_FLOW) {
-    grad_pairs(crho, sh, grx, gry);
-    grad_pairs(cp, sb, gpx, gpy);
+    grad_pairs<R, PIN>(crho, sh, grx, gry);
+    grad_pairs<R, PIN>(cp, sb, gpx, gpy);
   }
-  gphx *= R(3); gphy *= R(3); lphi *= R(3); lphi0 *= R(3); lfs *= R(3);
-  grx *= R(3); gry *= R(3); gpx *= R(3); gpy *= R(3);
+  gphx *= R(3); gphy *= R(3);
+  if constexpr (!PIN) lphi *= R(3);
+  lphi0 *= R(3); lfs *= R(3);
+  grx *= R(3); gry *= R(3);
+  if constexpr (!PIN) {
+    gpx *= R(3); gpy *= R(3);
+  }
 
   const R phi = L.phi, fs = L.fs, rho = L.rho, mdot = L.mdot;
   M.muphi = R(0);
@@ -389,13 +403,22 @@ __device__ __forceinline__ void node_macros(const Geom& g, const Coef<R>& c, int
   {
     R Fsx = R(0), Fsy = R(0);
     if (lat & LAT_PHASE) {
-      M.muphi = chem_local(c, phi, phi0, fs) -
-                c.klap * (lphi + c.cos_th * lphi0 + c.cos_ps * lfs);
+      if constexpr (PIN)
+        M.muphi = chem_local<R, true>(c, phi, phi0, fs) -
+                  c.klap * (sum2<1, R>(R(3), lphi, c.cos_th, lphi0) + c.cos_ps * lfs);
+      else
+        M.muphi = chem_local(c, phi, phi0, fs) -
+                  c.klap * (lphi + c.cos_th * lphi0 + c.cos_ps * lfs);
       Fsx = M.muphi * gphx;
       Fsy = M.muphi * gphy;
     }
-    Fx = Fsx + rho * c.gx;
-    Fy = Fsy + rho * c.gy;
+    if (PIN && (lat & LAT_PHASE)) {
+      Fx = sum2<P1, R>(M.muphi, gphx, rho, c.gx);
+      Fy = sum2<P1, R>(M.muphi, gphy, rho, c.gy);
+    } else {
+      Fx = Fsx + rho * c.gx;
+      Fy = Fsy + rho * c.gy;
+    }
   }
   M.ux = R(0); M.uy = R(0); M.uu = R(0); M.pr = R(0);
   if (lat & LAT_FLOW) {
@@ -451,12 +474,17 @@ __device__ __forceinline__ void node_macros(const Geom& g, const Coef<R>& c, int
       M.ux = usx + R(0.5) * fpx;
       M.uy = usy + R(0.5) * fpy;
     }
-    M.uu = M.ux * M.ux + M.uy * M.uy;
-    M.S = rho * mdot + M.ux * grx + M.uy * gry;
+    M.uu = sum2<P1, R>(M.ux, M.ux, M.uy, M.uy);
+    M.S = sum2<P1, R>(rho, mdot, M.ux, grx) + M.uy * gry;
     // modified force (reading R-FT), lagged pressure (reading R-FP)
-    M.Ftx = Fx - (gpx - grx * R(1.0 / 3.0));
-    M.Fty = Fy - (gpy - gry * R(1.0 / 3.0));
-    M.uFt = M.ux * M.Ftx + M.uy * M.Fty;
+    if constexpr (PIN) {
+      M.Ftx = Fx - sum2<1, R>(R(3), gpx, -grx, R(1.0 / 3.0));
+      M.Fty = Fy - sum2<1, R>(R(3), gpy, -gry, R(1.0 / 3.0));
+    } else {
+      M.Ftx = Fx - (gpx - grx * R(1.0 / 3.0));
+      M.Fty = Fy - (gpy - gry * R(1.0 / 3.0));
+    }
+    M.uFt = sum2<P1, R>(M.ux, M.Ftx, M.uy, M.Fty);
     if constexpr (WB) {
       // tau_f = 3 mu / rho + 1/2 rounded once (with the velocity above but
       // tau_f from two roundings the Stefan velocity stays at 1.2e-4; the
@@ -537,8 +565,14 @@ __device__ __forceinline__ void diag_values(const Coef<R>& c, int lat, const Loc
 // its grid).  LATC: compile-time lattice set (7 = all three) or 0 (read at
 // run time).  FEW: a float step's phase B in the form of lbm_wb.cuh.  Every
 // thread of the CTA calls it.
+//
+// RW: warps beyond the tile's own that take the ring (a ring node a thread)
+// while the tile's warps take its nodes.  A double column's tile is one warp
+// (32 x 1) and a step lasts as long as that warp's chain of FP64 latencies;
+// its 70 ring nodes would be three more rounds of loads and of the local
+// state (512 x 8: 42 us a step, 30 with the ring on warps of its own).
 template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY,
-          bool FEW = false>
+          bool FEW = false, int RW = 0>
 __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, int b, int nb) {
   // the tile's shape; these hide the namespace's 32 x 8 constants
   constexpr int TY = Shape<TYS>::TY, HN = Shape<TYS>::HN, NT = Shape<TYS>::NT;
@@ -621,7 +655,48 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     s_rsg[k][part] = sgp;
     s_rsh[k][part] = shp;
   };
-  if constexpr (RING * NPART <= NT) {
+  if constexpr (RW > 0) {
+    static_assert(RING <= RW * TX && !WB, "a ring node a thread, plain storage");
+    if (ty >= TYS) {
+      const int k = tid - NT;
+      if (k < RING) {
+        int hx, hy;
+        ring_pos<TYS>(k, hx, hy);
+        const int hi = hy * HX + hx;
+        const int m = wrap_or_clamp(y0 + hy - 1, g.ny, g.bc[2], g.bc[3]) * g.pitch +
+                      wrap_or_clamp(x0 + hx - 1, g.nx, g.bc[0], g.bc[1]);
+        const S* pm = a.pin + m;
+        const R q0 = a.phi0[m], flq = a.lin[LAG_FL * P + m], wq = a.lin[LAG_W * P + m];
+        const R Qq = a.lin[LAG_Q * P + m], pq = a.lin[LAG_P * P + m];
+        R sgq = R(0), shq = R(0);
+        if (lat & LAT_PHASE) {
+          R v[9];
+#pragma unroll
+          for (int i = 0; i < 9; i++) v[i] = ldp(pm + (9 + i) * P);
+          sgq = sum_g(v);
+        }
+        if (lat & LAT_HEAT) {
+          R v[9];
+          if (g.has_mask && a.mask[m]) {
+            cold_mask_h(c, wq, q0, v);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 9; i++) v[i] = ldp(pm + (18 + i) * P);
+          }
+          shq = sum_h(v);
+        }
+        const Local<R> Lq = local_state(c, lat, sgq, shq, flq, wq, Qq, q0);
+        s_phi[hi] = Lq.phi;
+        s_fs[hi] = Lq.fs;
+        s_rho[hi] = Lq.rho;
+        s_p[hi] = pq;
+        s_phi0[hi] = q0;
+      }
+      __syncthreads();
+      if (DIAG) __syncthreads();  // the barrier of block_diag_finish
+      return;
+    }
+  } else if constexpr (RING * NPART <= NT) {
     if (tid < RING * NPART) ring_load(tid);
   } else {
     for (int job = tid; job < RING * NPART; job += NT) ring_load(job);
@@ -748,12 +823,13 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
     s_rho[hi] = Lq.rho;
     if constexpr (WB) s_T[hi] = Lq.T;
   };
-  if constexpr (RING <= NT) {
+  if constexpr (RW > 0) {
+  } else if constexpr (RING <= NT) {
     if (tid < RING) ring_state(tid);
   } else {
     for (int k = tid; k < RING; k += NT) ring_state(k);
   }
-  __syncthreads();
+  if (RW == 0) __syncthreads();
   if (MODE == MODE_STEP) allow_next();
 
   // ---- phase B: stencils, macros, collisions, streaming -------------------
@@ -821,11 +897,11 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
    }
   };
   auto phase_b = [&](auto interior) {
-  constexpr bool IN = decltype(interior)::value;
   if constexpr (FEW) {
     phase_b_few(interior);
     return;
   } else {
+  constexpr bool IN = decltype(interior)::value;
   R dvals[NDIAG];
   Macro<R> M;
   // links that stay inside the grid need no boundary logic
@@ -951,12 +1027,12 @@ __device__ __forceinline__ void step_tile(const Args<R, S>& a, int bx, int by, i
 // One CTA per 32 x TYS tile; float kernels keep the 64-register budget of
 // the 32 x 8 shape (4 CTAs of 256 threads per SM) at every shape.
 template <typename R, int MODE, bool DIAG, int LATC, typename S = R, int TYS = TY,
-          bool FEW = false>
-__global__ void __launch_bounds__(Shape<TYS>::NT,
+          bool FEW = false, int RW = 0>
+__global__ void __launch_bounds__(Shape<TYS>::NT + RW * TX,
                                   sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 * TY / TYS : 1)
     lbm_step_kernel(const Args<R, S> a) {
   after_previous();
-  step_tile<R, MODE, DIAG, LATC, S, TYS, FEW>(a, blockIdx.x, blockIdx.y, -1, 0);
+  step_tile<R, MODE, DIAG, LATC, S, TYS, FEW, RW>(a, blockIdx.x, blockIdx.y, -1, 0);
 }
 
 // Many independent grids (uneven sizes and parameters) advanced in one
@@ -975,8 +1051,8 @@ struct BatchTable {
   Args<R> args[BATCH_MAX_GRIDS];
 };
 
-template <typename R, bool DIAG, int LATC, int TYS = TY, bool FEW = false>
-__global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
+template <typename R, bool DIAG, int LATC, int TYS = TY, bool FEW = false, int RW = 0>
+__global__ void __launch_bounds__(Shape<TYS>::NT + RW * TX, sizeof(R) == 4 ? LBM_MIN_BLOCKS_F32 : 1)
     lbm_batch_kernel(const __grid_constant__ BatchTable<R> B) {
   after_previous();
   const int t = blockIdx.x;
@@ -990,8 +1066,8 @@ __global__ void __launch_bounds__(Shape<TYS>::NT, sizeof(R) == 4 ? LBM_MIN_BLOCK
   const int local = t - B.tile_base[lo];
   const int tiles_x = (a.g.nx + TX - 1) / TX;
   const int ntiles = B.tile_base[lo + 1] - B.tile_base[lo];
-  step_tile<R, MODE_STEP, DIAG, LATC, R, TYS, FEW>(a, local % tiles_x, local / tiles_x, local,
-                                                   ntiles);
+  step_tile<R, MODE_STEP, DIAG, LATC, R, TYS, FEW, RW>(a, local % tiles_x, local / tiles_x, local,
+                                                       ntiles);
 }
 
 }  // namespace lbmk
