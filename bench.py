@@ -142,13 +142,14 @@ def measured_peak():
 
 
 # the sources the step kernels are compiled from (host API and probes excluded)
-KERNEL_SOURCES = ("lbm_kernels.cuh", "lbm_dual.cuh", "lbm_step.cuh", "lbm_split.cuh",
-                  "lbm_tile.cuh", "lbm_tma.cuh", "lbm_launch.h", "lbm_f32.cu", "lbm_f64.cu",
-                  "lbm_f16.cu", "lbm_tan.cu")
+KERNEL_SOURCES = ("lbm_kernels.cuh", "lbm_dual.cuh", "lbm_pdl.cuh", "lbm_step.cuh", "lbm_wb.cuh",
+                  "lbm_column.cuh", "lbm_node.cuh", "lbm_tile.cuh", "lbm_tma.cuh", "lbm_launch.h",
+                  "lbm_f32.cu", "lbm_f64.cu", "lbm_f16.cu", "lbm_tan.cu", "lbm_node.cu")
 
 
 # the sources of the 3-D step kernels
-KERNEL_SOURCES3 = ("lbm3d.cu", "lbm_kernels.cuh", "lbm_dual.cuh", "lbm_host.h")
+KERNEL_SOURCES3 = ("lbm3d.cu", "lbm_node.cuh", "lbm_pdl.cuh", "lbm_kernels.cuh", "lbm_dual.cuh",
+                   "lbm_host.h")
 
 
 def kernel_source_hash(sources=KERNEL_SOURCES) -> str:
@@ -157,6 +158,15 @@ def kernel_source_hash(sources=KERNEL_SOURCES) -> str:
         with open(os.path.join(ROOT, "paper_2510_18688_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def kernels_per_step(precision: str, wls) -> int:
+    """Two in double and tangents (local states, then collisions), one in
+    float and in double columns (fewer than 32 rows)."""
+    if precision == "tangent":
+        return 2
+    column = wls[0][0]["ny"] < 32 and wls[0][0]["nx"] >= 4 * wls[0][0]["ny"]
+    return 2 if precision == "fp64" and not column else 1
 
 
 def profile_name(workload: str, precision: str) -> str:
@@ -739,10 +749,10 @@ def main():
     if batch is None and not args.no_autotune:
         us, chosen = solvers[0].autotune(64)
         tune = {"chosen": chosen, "us_per_step": us,
-                "variants": "kernel form v//2 (0 one CTA per 32x8 tile; 1 float TMA-staged "
-                            "one stage / fp64 two-kernel split; 2 TMA-staged two stages "
+                "variants": "kernel form v//2 (0 the default for the grid; 1 float TMA-staged "
+                            "one stage / fp64 node step, two kernels; 2 TMA-staged two stages "
                             "2 CTAs/SM; 3 TMA-staged one stage 3 CTAs/SM; 4 one CTA per "
-                            "32x4 tile; 5 one CTA per 32x16 tile; -1: not available) x "
+                            "32x4 tile; 5 one CTA per 32x16 (fp64 32x2) tile; -1: not available) x "
                             "captured period (v even 32, odd 256); timed back to back "
                             "without L2 flush"}
 
@@ -888,7 +898,7 @@ def main():
                    "parallelism": f"replicas x{world}"},
         "roofline": roofline,
         "autotune": tune,
-        "gpu_launches": args.steps,
+        "gpu_launches": args.steps * kernels_per_step(args.precision, wls),
         "e2e": e2e,
         "l2_resident_mlups": n / (l2_ms * 1e-3) / 1e6,
         "diag_last": {k: diag[k] for k in ("material_mass", "frozen_volume", "nonfinite", "step")},

@@ -140,14 +140,6 @@ __device__ __forceinline__ void cold_mask_h19(const Coef<R>& c, R w, R phi0, R* 
   for (int i = 1; i < Q; i++) h[i] = wq<R>(i) * rrT;
 }
 
-template <typename R>
-__device__ __forceinline__ R sum19(const R* v) {
-  R s = v[0];
-#pragma unroll
-  for (int i = 1; i < Q; i++) s += v[i];
-  return s;
-}
-
 // ---------------------------------------------------------------------------
 // the step and the read-out: the node kernels of lbm_node.cuh.  Float takes
 // 32 x 4 x 2 blocks, whose stencil halos stay in L1; double and tangents,

@@ -58,12 +58,12 @@ struct Shape {
 };
 __host__ __device__ constexpr int tiles_y(int ny, int ty) { return (ny + ty - 1) / ty; }
 // One-dimensional columns: fewer than 32 rows, at least four times as long,
-// at most 32768 nodes.  They stay with the fused tile from global loads.  In
-// double the node step is the faster one there too (512 x 8: 14.6 us a step;
-// fused 57 us on 32 x 8 tiles, 19 us on 32 x 1 with four warps), in float the TMA-staged tile
-// takes as long (9 us, latency alone); but across a column the velocity is
-// nothing but rounding (1e-20 against 4e-5 along it), and the fused tile keeps
-// every bit of it as earlier results and saved runs have it.
+// at most 32768 nodes.  They keep the arithmetic of the fused tile from global
+// loads (in double on four warps a tile, lbm_column.cuh).  The node step
+// (512 x 8 double: 14.3 us a step against 19) and the TMA-staged tile (float:
+// 9 us, latency alone, as the fused tile) would do; but across a column the
+// velocity is nothing but rounding (1e-20 against 4e-5 along it), and the
+// fused tile keeps every bit of it as earlier results and saved runs have it.
 __host__ __device__ inline bool is_column(int nx, int ny) {
   return ny < 32 && nx >= 4 * ny && (long long)nx * ny <= 32768;
 }
@@ -622,22 +622,18 @@ __device__ __forceinline__ void block_diag_warps(const R* dvals, R (*s_red)[NDIA
 }
 
 // Stage 2 (every thread; one barrier): the warps' sums in order into
-// partial[k * nb + b] for tile b of nb.
+// partial[k * nb + b] for tile b of nb.  In float the warps' sums are added
+// with Knuth's TwoSum (the rounding error of every addition is carried along
+// and added back at the end), so one conversion to double per diagnostic keeps
+// the accuracy of a double-precision sum without work on the slow FP64 pipe.
+// The grid-wide sum is lbm_diag_finalize_kernel.
 template <typename R, int NW = NT / 32>
 __device__ __forceinline__ void block_diag_finish(const R (*s_red)[NDIAG],
                                                   double* __restrict__ partial, int tid, int b,
                                                   int nb) {
   __syncthreads();
   if (tid < NDIAG) {
-    if constexpr (is_dual<R>::value) {
-      // tangent step: values in the first NDIAG * nb partials, derivatives
-      // in the next NDIAG * nb
-      R acc = R(0);
-#pragma unroll
-      for (int w = 0; w < NW; w++) acc += s_red[w][tid];
-      partial[(long long)tid * nb + b] = acc.v;
-      partial[(long long)(NDIAG + tid) * nb + b] = acc.d;
-    } else if constexpr (sizeof(R) == 8) {
+    if constexpr (sizeof(R) == 8) {
       double acc = 0.0;
 #pragma unroll
       for (int w = 0; w < NW; w++) acc += (double)s_red[w][tid];
@@ -655,29 +651,6 @@ __device__ __forceinline__ void block_diag_finish(const R (*s_red)[NDIAG],
       partial[(long long)tid * nb + b] = (double)sum + (double)err;
     }
   }
-}
-
-// Per-tile partial sums of the diagnostics in a fixed order (warp sums, then
-// the warps in order), written to partial[k * nb + b] for tile b of nb.
-// Every thread of the CTA calls it; s_red is shared memory of the arithmetic
-// type.  In float the warps' sums are added with Knuth's TwoSum (the
-// rounding error of every addition is carried along and added back at the
-// end), so one conversion to double per diagnostic keeps the accuracy of a
-// double-precision sum without work on the slow FP64 pipe.  The grid-wide
-// sum is lbm_diag_finalize_kernel.
-template <typename R>
-__device__ __forceinline__ void block_diag(const R* dvals, R (*s_red)[NDIAG],
-                                           double* __restrict__ partial, int tid, int b, int nb) {
-  block_diag_warps(dvals, s_red, tid);
-  block_diag_finish(s_red, partial, tid, b, nb);
-}
-
-// Single-grid launch: the tile is the CTA.
-template <typename R>
-__device__ __forceinline__ void block_diag(const R* dvals, R (*s_red)[NDIAG],
-                                           double* __restrict__ partial, int tid) {
-  block_diag(dvals, s_red, partial, tid, blockIdx.y * gridDim.x + blockIdx.x,
-             gridDim.x * gridDim.y);
 }
 
 // Grid-wide FP64 diagnostics from the partial sums (nb per diagnostic, one

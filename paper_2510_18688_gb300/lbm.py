@@ -294,7 +294,7 @@ def lbm_adjoint_coupled(ctx, nsteps: int, every: int, observable: int, axis: int
 
 
 # kernel form ids of lbm_autotune (variant v = form v // 2, period v % 2)
-FORMS = ("float: one CTA per 32x8 tile / fp64: by the grid",
+FORMS = ("by the grid",
          "float: TMA-staged, one stage / fp64: node kernels",
          "float: TMA-staged, two stages, 2 persistent CTAs per SM",
          "float: TMA-staged, one stage, 3 persistent CTAs per SM", "one CTA per 32x4 tile",
