@@ -1571,7 +1571,7 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   };
   // Where every state fits in an eighth of the free memory (LBM_ADJOINT_KEEP=0:
   // never) all are kept and none is computed twice: 48 steps of the 256 x 256
-  // droplet take 0.9 GB and 7.9 ms against 10.3 ms with a checkpoint every 16
+  // droplet take 0.9 GB and 7.6 ms against 9.1 ms with a checkpoint every 16
   // steps.  The states, and so the results, are the same.
   size_t freeb = 0, totalb = 0;
   cudaError_t e = cudaMemGetInfo(&freeb, &totalb);
