@@ -1,8 +1,8 @@
 // lbm_tile.cuh -- the fused time step of float states (FP32 and FP16
 // storage) as a persistent kernel whose tiles are staged by TMA, for sm_103a.
 //
-// The arithmetic is that of step_tile (lbm_step.cuh, well-balanced storage);
-// what differs is how a tile's inputs arrive.  Each CTA owns a sequence of
+// The phases are those of step_tile (lbm_step.cuh, well-balanced storage), phase
+// B in the form of lbm_wb.cuh; what differs is how a tile's inputs arrive.  Each CTA owns a sequence of
 // 32 x 8 tiles (blockIdx.x, blockIdx.x + gridDim.x, ...).  One thread issues
 // the TMA copies of the next tile's inputs into the free one of two
 // shared-memory stages while the CTA computes the current tile from the
@@ -462,8 +462,9 @@ __device__ __forceinline__ void tile_once(const Args<float, S>& a, const CUtenso
 
 // CTAs per SM of the loop-free one-stage kernels: four for one grid (64
 // registers, 56 KB of shared memory each); three for the batched kernel,
-// whose grid lookup does not fit 64 registers without spills (at four it
-// measured 632 us per step of the 64-grid batch against 610 us at three).
+// whose grid lookup does not fit 64 registers without spills (at four an
+// earlier phase B measured 632 us per step of the 64-grid batch against 610 us
+// at three; the present one takes 511 us at three).
 constexpr int kTileOnceBlocks = 4;
 constexpr int kTileBatchBlocks = 3;
 
