@@ -460,13 +460,12 @@ __device__ __forceinline__ void tile_once(const Args<float, S>& a, const CUtenso
   tile_step<S, DIAG, LATC>(a, stage[0], bx, by, b, nb, s_phi, s_wet, s_rho, s_T, s_red, mk);
 }
 
-// CTAs per SM of the loop-free one-stage kernels: four for one grid (64
-// registers, 56 KB of shared memory each); three for the batched kernel,
-// whose grid lookup does not fit 64 registers without spills (at four an
-// earlier phase B measured 632 us per step of the 64-grid batch against 610 us
-// at three; the present one takes 511 us at three).
+// CTAs per SM of the loop-free one-stage kernels: four, at 64 registers and
+// 56 KB of shared memory each.  The batched kernel's grid lookup fits too
+// since phase B holds less (8 B spilled): a step of the 64-grid batch takes
+// 473 us at four against 514 at three.
 constexpr int kTileOnceBlocks = 4;
-constexpr int kTileBatchBlocks = 3;
+constexpr int kTileBatchBlocks = 4;
 
 // One grid, one CTA per tile, one stage (kernel form 1).
 template <typename S, bool DIAG, int LATC>
