@@ -193,7 +193,12 @@ __device__ __forceinline__ MacroWb macros_wb(const Coef<float>& c, int lat, cons
     float t = fmaf(0.5f, M.S, snz);
     t = fmaf((4.f / 9.f) * (M.tauf - 0.5f), F0, t);
     t = fmaf((4.f / 9.f) * -1.5f * rho, M.uu, t);
-    const float dp = 0.6f * t;
+    // 1 / (3 (1 - w_0)) of the float weights, 0.59999996: the references
+    // 3 w_i p hold the same weights, and the pressure is the sum of these
+    // increments over the whole run.  With float(3/5), 1e-7 above it, p is
+    // 17 % and u 14-16 % further off on porous grids (36 states of 8 to 160
+    // steps against the 64-bit solution).
+    const float dp = ((1.f / 3.f) / (1.f - 4.f / 9.f)) * t;
     M.pr = pp + dp;
     const float bb = M.pr - pp;
     M.prl = (pp - (M.pr - bb)) + (dp - bb);

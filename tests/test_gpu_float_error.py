@@ -1,0 +1,48 @@
+"""The float step's error against the 64-bit oracle.  Its collisions are written
+with few products (lbm_wb.cuh); the form with one product after the other
+(node_macros and collide_*_wb of lbm_step.cuh) sets the bar: on the grids
+below its errors have the geometric means of LONG_FORM, and the short form
+may not be further off."""
+import numpy as np
+import pytest
+
+from paper_2510_18688_gb300 import workloads as W
+
+LONG_FORM = {"p": 6.361e-7, "ux": 5.851e-7, "uy": 6.655e-7}
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from oracle import oracle as O
+    from paper_2510_18688_gb300 import build, lbm
+    build.build()
+    lbm.load()
+    return O, lbm
+
+
+@pytest.fixture(scope="module")
+def porous_errors(env):
+    """Geometric mean over twelve porous grids of the relative L2 errors at
+    steps 8, 64 and 160, by field."""
+    O, lbm = env
+    logs = {k: [] for k in LONG_FORM}
+    for seed in range(12):
+        wl = W.porous(240 + seed, 170, seed=seed)
+        o = O.from_workload(wl)
+        s = lbm.Solver(wl[0], precision="fp32").set_geometry(wl[1])
+        for n in (8, 56, 96):
+            ref, got = o.step(n).fields(), s.step(n).fields()
+            for k in logs:
+                logs[k].append(np.log(np.linalg.norm(got[k] - ref[k]) / np.linalg.norm(ref[k])))
+        s.close()
+        o.close()
+    return {k: float(np.exp(np.mean(v))) for k, v in logs.items()}
+
+
+# the mean of 36 such errors varies by about 1 % with the order of roundings
+@pytest.mark.gpu
+def test_pressure_error_in_a_porous_medium(porous_errors):
+    assert porous_errors["p"] <= 1.05 * LONG_FORM["p"]
