@@ -361,10 +361,16 @@ cudaError_t launch(lbm_ctx* c, int mode, bool diag, double* const* outs, cudaStr
   return lbmk::launch_step_f16s(a, mode, diag, s, ty);
 }
 
-// One FP64 step from the state at pops / lags into pops1 / lags1 by the
-// context's own kernel, with the node step's planes in `planes`.
-cudaError_t step_between(lbm_ctx* c, double* pops, double* lags, double* pops1, double* lags1,
-                         double* planes, cudaStream_t s) {
+// Whether step number k reduces the sums.
+bool sums_at(const lbm_ctx* c, int64_t k) {
+  return c->p.diag_every > 0 && k % c->p.diag_every == 0;
+}
+
+// FP64 step number k from the state at pops / lags into pops1 / lags1 by the
+// kernel that lbm_step takes for it (a column's steps with and without sums
+// round differently), with the node step's planes in `planes`.
+cudaError_t step_between(lbm_ctx* c, int64_t k, double* pops, double* lags, double* pops1,
+                         double* lags1, double* planes, cudaStream_t s) {
   void* const keep[5] = {c->pop[0], c->pop[1], c->lag[0], c->lag[1], c->scratch};
   const int cur = c->cur;
   c->cur = 0;
@@ -373,7 +379,7 @@ cudaError_t step_between(lbm_ctx* c, double* pops, double* lags, double* pops1, 
   c->lag[0] = lags;
   c->lag[1] = lags1;
   c->scratch = planes;
-  const cudaError_t e = launch(c, lbmk::MODE_STEP, false, nullptr, s);
+  const cudaError_t e = launch(c, lbmk::MODE_STEP, sums_at(c, k), nullptr, s);
   c->pop[0] = keep[0];
   c->pop[1] = keep[1];
   c->lag[0] = keep[2];
@@ -418,7 +424,7 @@ void note_diag_span(lbm_ctx* c, int64_t first, int64_t end) {
 
 cudaError_t step_launches(lbm_ctx* c, int64_t nsteps, cudaStream_t s) {
   for (int64_t k = 0; k < nsteps; k++) {
-    const bool diag = c->p.diag_every > 0 && (c->step % c->p.diag_every) == 0;
+    const bool diag = sums_at(c, c->step);
     cudaError_t e = launch(c, lbmk::MODE_STEP, diag, nullptr, s);
     if (e != cudaSuccess) return e;
     note_diag_span(c, c->step, c->step + 1);
@@ -1621,12 +1627,13 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
       r = cudaMemcpyAsync(dst + pN, lags, lN * sizeof(double), cudaMemcpyDeviceToDevice, s);
     return r;
   };
-  // states 1 ... len - 1 of a segment from its first, each step straight into
+  // states 1 ... len - 1 of segment q from its first, each step straight into
   // its own slot
-  auto fill = [&](int64_t len) {
+  auto fill = [&](int64_t q, int64_t len) {
     cudaError_t r = cudaSuccess;
     for (int64_t j = 0; j + 1 < len && r == cudaSuccess; j++)
-      r = step_between(c, slot(j), slot(j) + pN, slot(j + 1), slot(j + 1) + pN, planes(j), s);
+      r = step_between(c, step0 + q * every + j, slot(j), slot(j) + pN, slot(j + 1),
+                       slot(j + 1) + pN, planes(j), s);
     return r;
   };
   // forward: checkpoints, or every state
@@ -1639,9 +1646,9 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   // the last segment stays in its slots; its last step leads back into the context
   if (e == cudaSuccess && st == LBM_OK) {
     const int64_t len = nsteps - (nck - 1) * every;
-    e = fill(len);
+    e = fill(nck - 1, len);
     if (e == cudaSuccess)
-      e = step_between(c, slot(len - 1), slot(len - 1) + pN, (double*)c->pop[c->cur ^ 1],
+      e = step_between(c, step0 + nsteps - 1, slot(len - 1), slot(len - 1) + pN, (double*)c->pop[c->cur ^ 1],
                        (double*)c->lag[c->cur ^ 1], planes(len - 1), s);
     c->cur ^= 1;
     c->step += len;
@@ -1709,7 +1716,7 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
     const int64_t len = std::min<int64_t>(every, nsteps - q * every);
     if (q < nck - 1) {
       e = copy_state(slot(0), ck + q * stN, ck + q * stN + pN);
-      if (e == cudaSuccess) e = fill(len);
+      if (e == cudaSuccess) e = fill(q, len);
     }
     for (int64_t j = len - 1; j >= 0 && e == cudaSuccess; j--) {
       // the last state of a segment: the lags its step wrote are in the
@@ -2003,7 +2010,7 @@ cudaError_t batch_group(lbm_batch* b, const std::vector<lbm_ctx*>& list, int kin
 cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
   lbm_ctx* c0 = b->ctx[0];
   for (int64_t k = 0; k < nsteps; k++) {
-    const bool diag = c0->p.diag_every > 0 && (c0->step % c0->p.diag_every) == 0;
+    const bool diag = sums_at(c0, c0->step);
     // each grid by its own default kernel, as lbm_step takes it
     const bool f64 = b->precision == LBM_FP64;
     cudaError_t e =

@@ -141,6 +141,28 @@ def test_coupled_adjoint_with_all_states_equals_checkpoints(env, nx, ny, every, 
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(70, 12), (130, 5), (40, 33)])
+@pytest.mark.parametrize("diag_every", [1, 3])
+def test_coupled_adjoint_steps_as_lbm_step_with_sums(env, nx, ny, diag_every, monkeypatch):
+    """A context that reduces its sums every few steps (a column's kernels round
+    such steps differently): kept or recomputed states give one value, gradient
+    and final state, and that state is lbm_step's, bit for bit."""
+    _, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=3)
+    a, b, c = (lbm.Solver(cfg, precision="fp64", diag_every=diag_every).set_geometry(arr)
+               for _ in range(3))
+    va, ga, ta = a.adjoint_coupled(23, observable=0, every=5, initial_T=True)
+    monkeypatch.setenv("LBM_ADJOINT_KEEP", "0")
+    vb, gb, tb = b.adjoint_coupled(23, observable=0, every=5, initial_T=True)
+    assert va == vb and ga == gb and np.array_equal(ta, tb)
+    fa, fb, fc = a.fields(), b.fields(), c.step(23).fields()
+    for k in FIELDS:
+        assert np.array_equal(fa[k], fb[k]) and np.array_equal(fa[k], fc[k]), k
+    for s in (a, b, c):
+        s.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,nz", [(31, 4, 3), (32, 4, 2), (33, 5, 4), (64, 2, 3), (5, 43, 6)])
 @pytest.mark.parametrize("seed", [0, 3])
 def test_three_dimensional_sizes_match_the_oracle(env, nx, ny, nz, seed):
