@@ -197,8 +197,8 @@ int lbm_step(lbm_ctx* ctx, int64_t nsteps, void* stream);
 /* Writes the fields selected by field_mask for the current state (the
  * values the next step would compute before its collisions), as [ny][nx] doubles,
  * into out[k] for every selected bit k (out[k] may be NULL otherwise).
- * where = LBM_HOST copies through a context-owned device staging buffer and
- * synchronises `stream`. */
+ * where = LBM_HOST copies through a context-owned device staging buffer.
+ * Synchronises `stream`, with LBM_DEVICE too. */
 int lbm_read_fields(lbm_ctx* ctx, uint32_t field_mask, double* const* out, int where,
                     void* stream);
 

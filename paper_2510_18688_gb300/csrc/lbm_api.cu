@@ -262,11 +262,12 @@ void set_kernel_form(lbm_ctx* c, int form) {
 }
 
 // A tile kernel whose copies did not arrive within its bounded wait sets
-// *c->status (pinned host memory: no copy to read it); the next synchronising
-// read, and every read of a float context's fields, reports it (once).  The
-// kernels of double and tangent contexts wait for no copies.
+// *c->status (pinned host memory: no copy to read it); every read of fields,
+// into device memory too, and the next other synchronising read reports it
+// (once).  They wait for `s` in every precision, double and tangent contexts
+// included, whose kernels set no status: a read-out is complete, and a failed
+// kernel reported, when the call returns.
 int check_timeout(lbm_ctx* c, cudaStream_t s) {
-  if (!c->tile_ok) return LBM_OK;
   const cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(c, e, "synchronisation");
   volatile unsigned* v = c->status;

@@ -163,6 +163,25 @@ def test_coupled_adjoint_steps_as_lbm_step_with_sums(env, nx, ny, diag_every, mo
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp64", "tangent", "fp32", "fp16s"])
+def test_device_read_outs_are_complete_on_return(env, prec):
+    """Fields read into device memory can be taken on any stream, in every
+    precision: the call waits for the steps before it and for the read-out."""
+    import torch
+    _, lbm = env
+    cfg, arr = W.random_state(300, 200, seed=1)
+    s = lbm.Solver(cfg, precision=prec, tangent={"T_cold": 1.0} if prec == "tangent" else None)
+    s.set_geometry(arr).step(64)
+    torch.cuda.synchronize()
+    out = torch.empty((12, 200, 300), dtype=torch.float64, device="cuda")
+    ptrs = [out[k].data_ptr() for k in range(12)]
+    s.step(1024)
+    lbm.lbm_read_fields(s.ctx, 0xfff, ptrs, lbm.LBM_DEVICE, lbm._stream())
+    assert torch.cuda.current_stream().query()
+    s.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,nz", [(31, 4, 3), (32, 4, 2), (33, 5, 4), (64, 2, 3), (5, 43, 6)])
 @pytest.mark.parametrize("seed", [0, 3])
 def test_three_dimensional_sizes_match_the_oracle(env, nx, ny, nz, seed):
