@@ -435,10 +435,11 @@ int lbm_adjoint_coupled(lbm_ctx* ctx, int64_t nsteps, int every, int observable,
  * kernel form v / 2 with captured periods of at least 32 steps (v even) or
  * 256 (v odd).  Kernel forms (form ids; a context times those it has):
  * 0 float: as 1, on columns one CTA per 32 x 8 tile loading from global
- * memory (LBM_STEP_KERNEL=fused: everywhere), LBM_FP64 and tangents: the default, two node kernels of one thread per node (LBM_FP64
- * columns, fewer than 32 rows and at least four times as long: one CTA per
- * 32 x 1 tile); 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one
- * shared-memory stage and one CTA per tile, LBM_FP64: the node kernels; 2 (float) the
+ * memory (LBM_STEP_KERNEL=fused: everywhere), LBM_FP64 and tangents: two node
+ * kernels of one thread per node (LBM_FP64 columns -- fewer than 32 rows, at
+ * least four times as long, at most 32,768 nodes --: one CTA per 32 x 1 tile);
+ * 1 LBM_FP32/LBM_FP16S: the TMA-staged tile kernel with one shared-memory
+ * stage and one CTA per tile, LBM_FP64: the node kernels; 2 (float) the
  * TMA-staged kernel with two stages and two persistent CTAs per
  * multiprocessor (the copies of the next tile overlap the current one);
  * 3 (float) one stage and three persistent CTAs per multiprocessor; 4 one
@@ -454,7 +455,8 @@ int lbm_adjoint_coupled(lbm_ctx* ctx, int64_t nsteps, int every, int observable,
  * microseconds per step of each variant (-1 where not run); chosen (may be
  * NULL): the index kept.  The environment variable LBM_KERNEL_FORM=<form id>
  * read by lbm_create selects a form without timing (ignored where the
- * context does not have it).  Allocates a backup of the state (its population
+ * context does not have it); for LBM_FP64 so do LBM_STEP_KERNEL=split (form 1)
+ * and =fused (form 0 on columns, else form 4: one kernel a step).  Allocates a backup of the state (its population
  * and lag planes) for the duration of the call and synchronises `stream`.
  * Errors: LBM_ERR_ARG (steps_per_trial < 2), LBM_ERR_STATE before
  * lbm_set_geometry, LBM_ERR_OOM/LBM_ERR_CUDA. */

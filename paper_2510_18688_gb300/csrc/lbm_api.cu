@@ -638,6 +638,13 @@ int lbm_create(const lbm_params* params, lbm_ctx** out) {
       if (std::strcmp(k, "fused") == 0) form = 0;
     if (form >= 0) set_kernel_form(c, form);
   }
+  // LBM_STEP_KERNEL for FP64: `split` takes the two kernels of the node step on
+  // every grid, `fused` one kernel, which form 0 is on the columns alone
+  if (params->precision == LBM_FP64)
+    if (const char* k = std::getenv("LBM_STEP_KERNEL")) {
+      if (std::strcmp(k, "split") == 0) set_kernel_form(c, 1);
+      else if (std::strcmp(k, "fused") == 0 && c->node0) set_kernel_form(c, 4);
+    }
   // LBM_KERNEL_FORM=<form id> forces one kernel form where the context has it
   if (const char* f = std::getenv("LBM_KERNEL_FORM")) {
     char* end = nullptr;

@@ -182,6 +182,36 @@ def test_device_read_outs_are_complete_on_return(env, prec):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(130, 5), (53, 33)])
+def test_step_kernel_variable_selects_a_double_form(env, nx, ny, monkeypatch):
+    """LBM_STEP_KERNEL=split is the node step on columns too, =fused one kernel a
+    step on every grid: the states of the forms that the header names, bit for
+    bit, which on this state differ from the other kind's; all match the oracle."""
+    O, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=3)
+    ref = O.from_workload((cfg, arr)).step(40).fields()
+
+    def run(**env_vars):
+        for k, v in env_vars.items():
+            monkeypatch.setenv(k, v)
+        s = lbm.Solver(cfg, precision="fp64").set_geometry(arr)
+        for k in env_vars:
+            monkeypatch.delenv(k)
+        got = s.step(40).fields()
+        s.close()
+        _close(got, ref)
+        return got
+
+    def same(a, b):
+        return all(np.array_equal(a[k], b[k]) for k in FIELDS)
+
+    split, fused = run(LBM_STEP_KERNEL="split"), run(LBM_STEP_KERNEL="fused")
+    assert same(split, run(LBM_KERNEL_FORM="1"))
+    assert same(fused, run(LBM_KERNEL_FORM="0" if ny < 32 else "4"))
+    assert not same(split, fused)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,nz", [(31, 4, 3), (32, 4, 2), (33, 5, 4), (64, 2, 3), (5, 43, 6)])
 @pytest.mark.parametrize("seed", [0, 3])
 def test_three_dimensional_sizes_match_the_oracle(env, nx, ny, nz, seed):
