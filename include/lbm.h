@@ -311,10 +311,11 @@ void lbm_batch_destroy(lbm_batch* batch);
 
 /* Testing hook for the failure paths (host-side fault injection): with
  * after >= 0, the (after + 1)-th device or pinned-host allocation that
- * lbm_create makes from now on fails as if the device were out of memory
- * (lbm_create then returns LBM_ERR_OOM and frees what it had allocated);
- * the hook disarms itself after firing.  after < 0 disarms it.  Process
- * wide; not for concurrent use with other lbm_create calls. */
+ * lbm_create or lbm_adjoint_coupled makes from now on fails as if the device
+ * were out of memory (lbm_create then returns LBM_ERR_OOM and frees what it
+ * had allocated; lbm_adjoint_coupled keeps less); the hook disarms itself
+ * after firing.  after < 0 disarms it.  Process wide; not for concurrent use
+ * with other calls of the two. */
 void lbm_debug_fail_allocation(int after);
 
 /* Testing hook for the bounded waits of the float step's TMA-staged tile

@@ -111,9 +111,9 @@ struct StateHeader {
   int64_t step;
 };
 
-// Testing hook for the failure paths of lbm_create: when armed with n >= 0,
-// the (n + 1)-th device or pinned allocation made by lbm_create fails as if
-// the device were out of memory (then the hook disarms itself).
+// Testing hook for the failure paths of lbm_create and lbm_adjoint_coupled:
+// when armed with n >= 0, the (n + 1)-th device or pinned allocation they make
+// fails as if the device were out of memory (then the hook disarms itself).
 std::atomic<int> g_alloc_countdown{-1};
 
 // Testing hook for the bounded waits of the tile kernel: while armed, every
@@ -1575,8 +1575,9 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   // populations and lags, the stencil and local adjoints, the crossing seed,
   // the seed's lags and the accumulators; the states' fl and w, three field
   // planes, the sums.  A slot is a state and the planes of its local pass,
-  // which the reverse takes from the forward step.
-  const size_t slotN = stN + lbmn::NSC * P;
+  // which the reverse takes from the forward step; where that does not fit, a
+  // state alone, and the local pass is run again.
+  size_t slotN = stN + lbmn::NSC * P;
   const size_t clearN = 2 * stN + (lbmn::NSB + lbmn::NOWN + 1 + nacc) * P + lN;
   const size_t rest = clearN + (2 + 3) * P + 16;
   auto words = [&](int64_t ev) {
@@ -1598,7 +1599,7 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
     if (c->work) cudaFree(c->work);
     c->work = nullptr;
     c->work_len = 0;
-    const cudaError_t r = cudaMalloc((void**)&c->work, need * sizeof(double));
+    const cudaError_t r = dev_malloc((void**)&c->work, need * sizeof(double));
     if (r == cudaSuccess) c->work_len = need;
     else cudaGetLastError();  // not the next launch's error
     return r;
@@ -1606,6 +1607,10 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   e = cudaSuccess;
   if (all && reserve(words(nsteps)) != cudaSuccess) all = false;
   if (!all) e = reserve(words(every));
+  if (e == cudaErrorMemoryAllocation) {
+    slotN = stN;
+    e = reserve(words(every));
+  }
   if (e != cudaSuccess) return cuda_fail(c, e, "adjoint allocation");
   if (all) every = (int)std::min<int64_t>(nsteps, 1 << 30);
   const int64_t nck = (nsteps + every - 1) / every;
@@ -1628,7 +1633,8 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
   const int64_t step0 = c->step;
   e = cudaMemsetAsync(wk, 0, clearN * sizeof(double), s);
   auto slot = [&](int64_t j) { return seg + j * slotN; };
-  auto planes = [&](int64_t j) { return slot(j) + stN; };
+  const bool kept_planes = slotN > stN;
+  auto planes = [&](int64_t j) { return kept_planes ? slot(j) + stN : (double*)c->scratch; };
   auto copy_state = [&](double* dst, const double* pops, const double* lags) {
     cudaError_t r = cudaMemcpyAsync(dst, pops, pN * sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (r == cudaSuccess)
@@ -1729,7 +1735,7 @@ extern "C" int lbm_adjoint_coupled(lbm_ctx* c, int64_t nsteps, int every, int ob
     for (int64_t j = len - 1; j >= 0 && e == cudaSuccess; j--) {
       // the last state of a segment: the lags its step wrote are in the
       // context (last segment) or were not computed again
-      const bool last = j == len - 1, have = !last || q == nck - 1;
+      const bool last = j == len - 1, have = kept_planes && (!last || q == nck - 1);
       e = at_state(slot(j), slot(j) + pN, have ? planes(j) : nullptr,
                    last ? (double*)c->lag[c->cur] : slot(j + 1) + pN);
       set_io(cur_adj, cur_adj ^ 1);

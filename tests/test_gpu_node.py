@@ -163,6 +163,30 @@ def test_coupled_adjoint_steps_as_lbm_step_with_sums(env, nx, ny, diag_every, mo
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(70, 12), (40, 33)])
+def test_coupled_adjoint_runs_where_the_local_planes_do_not_fit(env, nx, ny, monkeypatch):
+    """Memory for the states alone is enough: an allocation with room for their
+    local planes that fails is followed by one without, and the results are the
+    same, bit for bit."""
+    _, lbm = env
+    cfg, arr = W.random_state(nx, ny, seed=4)
+    monkeypatch.setenv("LBM_ADJOINT_KEEP", "0")
+    a, b = (lbm.Solver(cfg, precision="fp64").set_geometry(arr) for _ in range(2))
+    va, ga, ta = a.adjoint_coupled(17, observable=0, every=5, initial_T=True)
+    lbm.lbm_debug_fail_allocation(0)
+    try:
+        vb, gb, tb = b.adjoint_coupled(17, observable=0, every=5, initial_T=True)
+        c = lbm.Solver(cfg, precision="fp64")  # the hook has fired: this one succeeds
+    finally:
+        lbm.lbm_debug_fail_allocation(-1)
+    assert va == vb and ga == gb and np.array_equal(ta, tb)
+    fa, fb = a.fields(), b.fields()
+    assert all(np.array_equal(fa[k], fb[k]) for k in FIELDS)
+    for s in (a, b, c):
+        s.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("prec", ["fp64", "tangent", "fp32", "fp16s"])
 def test_device_read_outs_are_complete_on_return(env, prec):
     """Fields read into device memory can be taken on any stream, in every
