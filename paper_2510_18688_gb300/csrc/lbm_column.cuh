@@ -1,6 +1,5 @@
 // lbm_column.cuh -- the double-precision step of thin columns (is_column) for
-// sm_103a: the arithmetic of step_tile, bit for bit, on 32 x 1 tiles with four
-// warps each.
+// sm_103a: the arithmetic of step_tile on 32 x 1 tiles with four warps each.
 //
 // A column has fewer tiles than the chip has SMs, so a step takes as long as
 // one tile does: a chain of FP64 latencies.  One warp a tile (step_tile on
@@ -14,9 +13,11 @@
 //
 // The bits: the compiler contracts a sum of two products one way or the
 // other, depending on the code around it, so every such sum whose order came
-// out differently here is written in step_tile's order (PIN, sum2).  A step
-// that reduces the sums is compiled to another order in places and stays with
-// step_tile, its ring on warps of its own (30 us).
+// out differently here on a one-dimensional column is written in step_tile's
+// order (PIN, sum2): the Neumann and Stefan columns have step_tile's bits.  A
+// state that varies across the column may differ from it in the last ones.  A
+// step that reduces the sums is compiled to another order in places and stays
+// with step_tile, its ring on warps of its own (30 us).
 #pragma once
 
 #include "lbm_step.cuh"

@@ -58,12 +58,17 @@ struct Shape {
 };
 __host__ __device__ constexpr int tiles_y(int ny, int ty) { return (ny + ty - 1) / ty; }
 // One-dimensional columns: fewer than 32 rows, at least four times as long,
-// at most 32768 nodes.  They keep the arithmetic of the fused tile from global
-// loads (in double on four warps a tile, lbm_column.cuh).  The node step
-// (512 x 8 double: 14.3 us a step against 19) and the TMA-staged tile (float:
-// 9 us, latency alone, as the fused tile) would do; but across a column the
-// velocity is nothing but rounding (1e-20 against 4e-5 along it), and the
-// fused tile keeps every bit of it as earlier results and saved runs have it.
+// at most 32768 nodes (a step of more fills the chip).  They keep the order of
+// operations of the fused tile from global loads (in double on four warps a
+// tile, lbm_column.cuh).  The node step (512 x 8 double: 14.3 us a step against
+// 19, or 30 with sums) and the TMA-staged tile (float: 9 us, latency alone, as
+// the fused tile) would do, with other last bits; but across a one-dimensional
+// column the velocity is nothing but rounding (1e-20 against 4e-5 along it), so
+// there other last bits are another field.  On the Neumann and Stefan columns
+// this form has every bit of the fused tile.  In double a state that varies
+// across agrees to rounding, a step that reduces the sums rounds differently
+// from one that does not, and forms chosen by lbm_autotune or by name take
+// their own order.
 __host__ __device__ inline bool is_column(int nx, int ny) {
   return ny < 32 && nx >= 4 * ny && (long long)nx * ny <= 32768;
 }
@@ -484,7 +489,6 @@ __device__ __forceinline__ Local<float> local_state_wb(const Coef<float>& c, int
   return L;
 }
 
-// Eq. (6) without the Laplacian terms.
 // a b + c d.  Which product of such a sum the compiler rounds before the FMA
 // is its own choice and changes with the code around it.  PIN = 1 rounds c d,
 // PIN = 2 rounds a b: a kernel that has to give the bits of an earlier one
@@ -496,6 +500,7 @@ __device__ __forceinline__ R sum2(R a, R b, R c, R d) {
   else return a * b + c * d;
 }
 
+// Eq. (6) without the Laplacian terms.
 template <typename R, bool PIN = false>
 __device__ __forceinline__ R chem_local(const Coef<R>& c, R phi, R phi0, R fs) {
   constexpr int P1 = PIN ? 1 : 0, P2 = PIN ? 2 : 0;

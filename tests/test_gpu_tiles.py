@@ -41,6 +41,25 @@ def test_columns_match_the_oracle(env, nx, ny, seed, diag_every):
     s.close()
 
 
+# the one-dimensional columns, whose velocity across is rounding alone: the four
+# warps a tile give every bit of step_tile, which forms 4 and 5 are
+@pytest.mark.gpu
+@pytest.mark.parametrize("wl", [W.neumann(400, 4), W.stefan(512, 8), W.stefan(300, 5)],
+                         ids=["neumann400x4", "stefan512x8", "stefan300x5"])
+def test_columns_keep_the_bits_of_the_fused_tile(env, wl, monkeypatch):
+    _, lbm = env
+    got = {}
+    for form in ("0", "4", "5"):
+        monkeypatch.setenv("LBM_KERNEL_FORM", form)
+        s = lbm.Solver(wl[0], precision="fp64").set_geometry(wl[1])
+        got[form] = [s.step(n).fields() for n in (1, 15, 184)]
+        s.close()
+    for form in ("4", "5"):
+        for x, y in zip(got["0"], got[form]):
+            for k in FIELDS:
+                assert np.array_equal(x[k], y[k]), (form, k)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("lattices", [1, 2, 4, 3, 5, 6, 7])
 def test_columns_lattice_sets_and_the_readings_variant(env, lattices):
