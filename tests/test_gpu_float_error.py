@@ -46,3 +46,20 @@ def porous_errors(env):
 @pytest.mark.gpu
 def test_pressure_error_in_a_porous_medium(porous_errors):
     assert porous_errors["p"] <= 1.05 * LONG_FORM["p"]
+
+
+@pytest.mark.gpu
+def test_pressure_error_of_a_fracture_after_256_steps(env):
+    """Three dimensions: a pressure factor one float above 1 / (3 (1 - w_0)) = 1/2
+    makes p drift by 2^-23 a step, 3.1e-5 in 256 steps.  The relative L2 error
+    stays below a third of that."""
+    from oracle import oracle3d as O3
+    O3.build()
+    _, lbm = env
+    for seed in range(3):
+        wl = W.rough_fracture(64, 64, 24, seed=seed)
+        o, s = O3.from_workload(wl), lbm.Solver3(wl[0], "fp32").set_geometry(wl[1])
+        ref, got = o.step(256).fields()["p"], s.step(256).fields()["p"]
+        assert np.linalg.norm(got - ref) <= 256 * 2.0 ** -23 / 3 * np.linalg.norm(ref)
+        s.close()
+        o.close()
