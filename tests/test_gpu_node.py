@@ -289,3 +289,48 @@ def test_third_order_reciprocal_is_within_an_ulp():
         q = _fma(_fma(-q0, b, a), x, q0)
         exact = Fraction(a) / Fraction(b)
         assert abs(Fraction(q) - exact) < Fraction(float(np.spacing(abs(float(exact)))))
+
+
+PROBE = r"""
+#include "lbm_node.cuh"
+__global__ void probe(const double* a, const double* b, double* r, double* q, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  r[i] = lbmn::rcp(b[i]);
+  q[i] = lbmn::quot(a[i], b[i]);
+}
+extern "C" int run_probe(const double* a, const double* b, double* r, double* q, int n) {
+  probe<<<(n + 255) / 256, 256>>>(a, b, r, q, n);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+@pytest.mark.gpu
+def test_device_reciprocal_and_quotient_are_within_an_ulp(env, tmp_path):
+    """rcp and quot of lbm_node.cuh on the device, hardware seed and all, against
+    the IEEE results: mantissas at and beside the powers of two, and random ones,
+    over exponents whose reciprocals and quotients are normal numbers."""
+    import ctypes
+    import subprocess
+
+    import torch
+    from paper_2510_18688_gb300 import build
+    (tmp_path / "probe.cu").write_text(PROBE)
+    so = tmp_path / "probe.so"
+    subprocess.run([build.nvcc(), build.ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
+                    "-I", build.SRC, str(tmp_path / "probe.cu"), "-o", str(so)], check=True)
+    r = np.random.default_rng(11)
+    n = 1 << 21
+    m = np.concatenate([r.uniform(1.0, 2.0, n), 1.0 + np.arange(4096) * 2.0 ** -52,
+                        2.0 - np.arange(1, 4097) * 2.0 ** -52, 1.0 + np.arange(8192) / 8192.0])
+    b = np.ldexp(m, r.integers(-500, 501, m.size))
+    a = np.ldexp(r.permutation(m), r.integers(-500, 501, m.size)) * r.choice([-1.0, 1.0], m.size)
+    ta, tb = (torch.as_tensor(v, device="cuda") for v in (a, b))
+    tr, tq = torch.empty_like(tb), torch.empty_like(tb)
+    torch.cuda.synchronize()
+    f = ctypes.CDLL(str(so)).run_probe
+    f.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int]
+    assert f(ta.data_ptr(), tb.data_ptr(), tr.data_ptr(), tq.data_ptr(), m.size) == 0
+    for got, want in ((tr.cpu().numpy(), 1.0 / b), (tq.cpu().numpy(), a / b)):
+        assert np.all(np.abs(got - want) <= np.spacing(np.abs(want)))
