@@ -160,13 +160,35 @@ def kernel_source_hash(sources=KERNEL_SOURCES) -> str:
     return h.hexdigest()[:16]
 
 
-def kernels_per_step(precision: str, wls) -> int:
-    """Two in double and tangents (local states, then collisions), one in
-    float and in double columns (fewer than 32 rows)."""
+def is_column(cfg: dict) -> bool:
+    """The library's rule (lbm_kernels.cuh)."""
+    nx, ny = cfg["nx"], cfg["ny"]
+    return ny < 32 and nx >= 4 * ny and nx * ny <= 32768
+
+
+def forced_form(precision: str, cfg: dict) -> int:
+    """The kernel form lbm_create takes: 0 unless the environment names one."""
+    form = 0
+    if precision == "fp64":
+        k = os.environ.get("LBM_STEP_KERNEL", "")
+        form = 1 if k == "split" else 4 if k == "fused" and not is_column(cfg) else 0
+    named = os.environ.get("LBM_KERNEL_FORM", "")
+    if named.isdigit() and int(named) in ((0, 1, 4, 5) if precision == "fp64" else range(6)):
+        form = int(named)
+    return form
+
+
+def kernels_per_step(precision: str, cfgs: list, form: int = 0) -> int:
+    """Kernels that one step launches.  Double and tangents: two (local states,
+    then collisions); double columns in form 0, and forms 4 and 5, one.  Float:
+    one.  Batches: so many for up to 64 grids, the columns apart."""
     if precision == "tangent":
         return 2
-    column = wls[0][0]["ny"] < 32 and wls[0][0]["nx"] >= 4 * wls[0][0]["ny"]
-    return 2 if precision == "fp64" and not column else 1
+    pair = 2 if precision == "fp64" else 1
+    if len(cfgs) > 1:
+        thin = sum(is_column(c) for c in cfgs)
+        return -(-(len(cfgs) - thin) // 64) * pair + -(-thin // 64)
+    return 1 if form in (4, 5) or (form == 0 and is_column(cfgs[0])) else pair
 
 
 def profile_name(workload: str, precision: str) -> str:
@@ -898,7 +920,9 @@ def main():
                    "parallelism": f"replicas x{world}"},
         "roofline": roofline,
         "autotune": tune,
-        "gpu_launches": args.steps * kernels_per_step(args.precision, wls),
+        "gpu_launches": args.steps * kernels_per_step(
+            args.precision, [c for c, _ in wls],
+            tune["chosen"] // 2 if tune else forced_form(args.precision, wls[0][0])),
         "e2e": e2e,
         "l2_resident_mlups": n / (l2_ms * 1e-3) / 1e6,
         "diag_last": {k: diag[k] for k in ("material_mass", "frozen_volume", "nonfinite", "step")},

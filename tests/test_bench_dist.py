@@ -47,3 +47,18 @@ def test_whole_job_throughput_is_the_sum_over_ranks():
     one = bench.whole_job_mlups(262144, 1, 100, 3.3)
     assert bench.whole_job_mlups(262144, 4, 100, 3.3) == pytest.approx(4 * one)
     assert bench.max_over_ranks(2.5, None) == 2.5
+
+
+@pytest.mark.parametrize("precision,sizes,form,kernels", [
+    ("fp32", [(512, 512)], 0, 1), ("fp16s", [(512, 512)], 4, 1), ("tangent", [(512, 8)], 0, 2),
+    ("fp64", [(512, 512)], 0, 2), ("fp64", [(512, 512)], 1, 2), ("fp64", [(512, 512)], 4, 1),
+    ("fp64", [(512, 512)], 5, 1), ("fp64", [(512, 8)], 0, 1), ("fp64", [(512, 8)], 1, 2),
+    ("fp64", [(4096, 16)], 0, 2), ("fp64", [(2048, 16)], 0, 1), ("fp64", [(124, 32)], 0, 2),
+    ("fp64", [(128, 128)] * 64 + [(512, 8)] * 65, 0, 4), ("fp32", [(128, 128)] * 65, 0, 2),
+    ("fp64", [(512, 8)] * 3, 0, 1)])
+def test_launches_a_step_follow_the_library_s_dispatch(precision, sizes, form, kernels):
+    """The node limit of the column rule, the form the autotuner keeps, and the
+    64 grids of a batched launch are all counted."""
+    import bench
+    cfgs = [dict(nx=nx, ny=ny) for nx, ny in sizes]
+    assert bench.kernels_per_step(precision, cfgs, form) == kernels
