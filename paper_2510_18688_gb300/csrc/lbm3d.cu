@@ -5,21 +5,21 @@
 // The model is the two-dimensional one with every lattice sum taken over the
 // 19 velocities and every vector carrying a z component (flow Eqs. (11),
 // (14)-(17); phase field Eqs. (18)-(22); enthalpy Eqs. (23)-(28); the
-// isotropic stencils built on the D3Q19 weights).  The lattice-independent
-// local physics (the inversion of Eq. (8), the mass source, the order
-// parameter, Eq. (10), the local part of Eq. (6)) is shared with the 2-D
-// step through lbm_kernels.cuh.
+// isotropic stencils built on the D3Q19 weights).  The step is that of
+// lbm_node.cuh, which serves both lattices; the initial state and the
+// diagnostics take the lattice-independent local physics of lbm_kernels.cuh.
 //
 // A step is the two node kernels of lbm_node.cuh over the whole grid: the
 // local state of every node, then stencils, collisions and streaming.  The
 // 2-D float step fuses both halves with a recomputed halo ring; in 3-D the
 // ring of a 256-node tile is 2.2 times the tile, so the split form moves
-// fewer bytes: eight local planes (32 B per node in FP32) instead of the
-// ring's population sums.
+// fewer bytes: six local planes, and f_l and w straight into the next lags
+// (32 B per node in FP32), instead of the ring's population sums.
 //
-// What bounds it: FP32 the HBM traffic of the two passes, 201 + 529 B a node
-// against 516 B of a single pass (256 x 128 x 30 nodes: 35 + 93 us, 83 % and
-// 82 % of the copy rate; the collisions written pair by pair with general
+// What bounds it: FP32 the memory traffic of the two passes, 201 + 529 B a node
+// against 516 B of a single pass, about 665 of the 730 B through DRAM and the
+// rest from L2 (256 x 128 x 30 nodes: 35 + 93 us, 83 % and 82 % of the copy rate
+// by the 730; the collisions written pair by pair with general
 // streaming code took 178 us, at 24 warps an SM bound by latency; these fit
 // 64 registers and 32 warps, at 24 they take 98 us).  Double:
 // the FP64 pipe (131 x 67 x 30 nodes: 47 + 244 us against 61 + 621 us).

@@ -284,7 +284,7 @@ static __global__ void __launch_bounds__(NT) lbm_adjoint_init_kernel(const AdjAr
 }
 #endif  // LBM_ADJOINT_KERNELS
 
-// Fixed-order sum of the accumulator planes over the grid (one CTA).
+// Fixed-order sum of the accumulator planes over the grid (one CTA a plane).
 #ifdef LBM_ADJOINT_KERNELS
 static __global__ void __launch_bounds__(RED_NT) lbm_adjoint_reduce_kernel(
     const double* __restrict__ acc, Geom g, double* __restrict__ out) {

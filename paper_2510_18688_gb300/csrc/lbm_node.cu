@@ -4,8 +4,9 @@
 
 namespace lbmn {
 
-// Up to 256 threads; 128 registers in double (two resident blocks of 256,
-// sixteen warps per SM, saturate the FP64 pipe), all 255 for a tangent.
+// The bound that sets the registers a thread, not a block's size (blocks have
+// 32 to 128 threads, warps_per_block): 128 registers in double, so that sixteen
+// warps fit an SM, which saturate its FP64 pipe; all 255 for a tangent.
 constexpr int NTN = 256;
 template <typename R>
 constexpr int min_blocks() {
@@ -34,7 +35,7 @@ __global__ void __launch_bounds__(NTN, min_blocks<R>())
   node_collide_linear<R, 2, LATC, true, DIAG, int>(a, &ro, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// Warps per block: four where that still gives every SM several blocks; a
+// Warps per block: four where that still gives each of GB300's 152 SMs several blocks; a
 // grid of a few thousand nodes is spread warp by warp, so that no SM gets
 // more than its share of the FP64 work.
 static int warps_per_block(int nwarps) {

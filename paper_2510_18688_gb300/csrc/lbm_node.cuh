@@ -219,7 +219,7 @@ struct NodeCoef {
   unsigned readings;
 };
 
-// Division of a node id by a grid extent: q = (id m) >> (32 + s) with the
+// Division of a node id by a grid extent: q = (id m) >> (31 + s) with the
 // round-up multiplier of Granlund and Montgomery, exact for 0 <= id < 2^31.
 struct FastDiv {
   unsigned d, m, s;
