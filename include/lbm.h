@@ -281,8 +281,10 @@ void lbm_destroy(lbm_ctx* ctx);
  * results agree to the last bit where the compiler contracts both kernels'
  * copies of the arithmetic alike, as the FP64 build does, and otherwise to a
  * few roundings of the working precision).  LBM_FP64 batches take two launches
- * per step and per 64 grids, and one more per 64 columns.  This is how
- * many small problems fill the GPU.  LBM_FP32 batches run as the batched
+ * per step and per 64 grids; columns (lbm_autotune) take one more per 64, in
+ * LBM_FP32 too, on a second stream of the batch's own that starts from and is
+ * joined to `stream` (on `stream` itself while that is being captured).  This is
+ * how many small problems fill the GPU.  LBM_FP32 batches run as the batched
  * TMA-staged tile kernel (each tile's inputs copied to shared memory by the
  * tensor copies of its own context, one CTA per 32 x 8 tile; a copy that
  * does not arrive within the bounded wait makes that context's next read

@@ -1916,6 +1916,10 @@ struct lbm_batch {
   lbmk::TileBatch<float>* ttab;
   lbmk::BatchTable<float>* ftab;
   cudaStream_t cap_stream;
+  // where a batch has both kinds of grids: the columns' launches run on `side`,
+  // beside the others' (made at the first step outside a caller's capture)
+  cudaStream_t side;
+  cudaEvent_t fork, join;
   cudaGraphExec_t graph;               // one captured period of batch steps
   std::vector<uint64_t> graph_key;     // (parity, generation) per context, phase
   char err[512];
@@ -2021,23 +2025,53 @@ cudaError_t batch_group(lbm_batch* b, const std::vector<lbm_ctx*>& list, int kin
   return cudaSuccess;
 }
 
-cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
+// The batch's second stream, if it has use for one (a failure leaves the two
+// groups one after the other on the caller's).
+void make_side(lbm_batch* b) {
+  if (b->side || b->wide.empty() || b->thin.empty()) return;
+  bool ok = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) == cudaSuccess;
+  if (ok) return;
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
+  b->fork = b->join = nullptr;
+  b->side = nullptr;
+  cudaGetLastError();
+}
+
+// beside: columns and other grids, which share nothing, on two streams from
+// here to the end of the steps.  Neither fills the chip as a rule, so their
+// latencies overlap; one after the other they add up.
+cudaError_t batch_launches(lbm_batch* b, int64_t nsteps, cudaStream_t s, bool beside) {
   lbm_ctx* c0 = b->ctx[0];
-  for (int64_t k = 0; k < nsteps; k++) {
+  cudaError_t e = cudaSuccess;
+  cudaStream_t st = s;
+  if (beside && b->side && nsteps > 0) {
+    e = cudaEventRecord(b->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->fork, 0);
+    if (e != cudaSuccess) return e;
+    st = b->side;
+  }
+  for (int64_t k = 0; k < nsteps && e == cudaSuccess; k++) {
     const bool diag = sums_at(c0, c0->step);
     // each grid by its own default kernel, as lbm_step takes it
     const bool f64 = b->precision == LBM_FP64;
-    cudaError_t e =
-        batch_group(b, b->wide, f64 ? BATCH_NODE : (b->tile ? BATCH_TILE : BATCH_FUSED), diag, s);
-    if (e == cudaSuccess) e = batch_group(b, b->thin, f64 ? BATCH_THIN : BATCH_COLUMN, diag, s);
-    if (e != cudaSuccess) return e;
+    e = batch_group(b, b->wide, f64 ? BATCH_NODE : (b->tile ? BATCH_TILE : BATCH_FUSED), diag, s);
+    if (e == cudaSuccess) e = batch_group(b, b->thin, f64 ? BATCH_THIN : BATCH_COLUMN, diag, st);
+    if (e != cudaSuccess) break;
     note_batch_diag(b, c0->step, 1);
     for (lbm_ctx* c : b->ctx) {
       c->cur ^= 1;
       c->step++;
     }
   }
-  return cudaSuccess;
+  if (st != s) {  // after an error too: what was launched is waited for
+    cudaError_t j = cudaEventRecord(b->join, st);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(s, b->join, 0);
+    if (e == cudaSuccess) e = j;
+  }
+  return e;
 }
 
 std::vector<uint64_t> batch_key(const lbm_batch* b, int period) {
@@ -2078,7 +2112,7 @@ cudaError_t batch_graph(lbm_batch* b, int period, cudaGraphExec_t* out) {
     saved.push_back({c->cur, c->step, c->diag_step, c->have_diag, c->diag_pending});
   e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  cudaError_t el = batch_launches(b, period, b->cap_stream);
+  cudaError_t el = batch_launches(b, period, b->cap_stream, true);
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(b->cap_stream, &g);
   for (size_t i = 0; i < b->ctx.size(); i++) {
@@ -2109,7 +2143,9 @@ int batch_step_impl(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
   int64_t left = nsteps;
   const int period = graph_period(c0->p.diag_every, c0->graph_min);
   cudaError_t e = cudaSuccess;
-  if (c0->graphs && period <= kMaxGraphSteps && left >= period && stream_free(s)) {
+  const bool free = stream_free(s);
+  if (free) make_side(b);
+  if (c0->graphs && period <= kMaxGraphSteps && left >= period && free) {
     cudaGraphExec_t g = nullptr;
     e = batch_graph(b, period, &g);
     if (e != cudaSuccess) {
@@ -2126,7 +2162,7 @@ int batch_step_impl(lbm_batch* b, int64_t nsteps, cudaStream_t s) {
     for (lbm_ctx* c : b->ctx) c->step += reps * period;  // even period: parities unchanged
     left -= reps * period;
   }
-  e = batch_launches(b, left, s);
+  e = batch_launches(b, left, s, free);
   for (lbm_ctx* c : b->ctx) c->last_stream = s;
   if (e != cudaSuccess) {
     std::snprintf(b->err, sizeof(b->err), "batch kernel launch: %s", cudaGetErrorString(e));
@@ -2197,6 +2233,9 @@ void lbm_batch_destroy(lbm_batch* b) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+  if (b->side) cudaStreamDestroy(b->side);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
   delete b->ntab;
   delete b->dtab;
   delete b->ttab;

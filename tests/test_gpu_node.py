@@ -163,6 +163,46 @@ def test_coupled_adjoint_steps_as_lbm_step_with_sums(env, nx, ny, diag_every, mo
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_batches_of_columns_and_other_grids(env, prec):
+    """The two groups advance side by side: however the steps are grouped into
+    calls, captured or not, on whichever stream, every context has the same
+    fields and sums, bit for bit, and work queued after the call sees them."""
+    import torch
+    _, lbm = env
+    wls = [W.random_state(nx, ny, seed=i)
+           for i, (nx, ny) in enumerate([(512, 8), (40, 33), (130, 5), (96, 70), (64, 2)])]
+
+    def solvers():
+        return [lbm.Solver(c, precision=prec, diag_every=4).set_geometry(a) for c, a in wls]
+
+    sets = [solvers() for _ in range(3)]
+    torch.cuda.synchronize()
+    b = lbm.Batch(sets[0])
+    b.step(100)
+    b.step(23)
+    one = lbm.Batch(sets[1])
+    for _ in range(123):
+        one.step(1)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        lbm.Batch(sets[2]).step(60).step(63)
+        got2 = [s.fields() for s in sets[2]]
+    got = [[s.fields() for s in ss] for ss in sets[:2]] + [got2]
+    sums = [[s.diagnostics(compute=False) for s in ss] for ss in sets]
+    for i in range(len(wls)):
+        for k in FIELDS:
+            assert np.array_equal(got[0][i][k], got[1][i][k]), (i, k)
+            assert np.array_equal(got[0][i][k], got[2][i][k]), (i, k)
+        assert sums[0][i] == sums[1][i] == sums[2][i]
+    for h in (b, one):
+        h.close()
+    for ss in sets:
+        for s in ss:
+            s.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny", [(70, 12), (40, 33)])
 def test_coupled_adjoint_runs_where_the_local_planes_do_not_fit(env, nx, ny, monkeypatch):
     """Memory for the states alone is enough: an allocation with room for their
