@@ -203,6 +203,26 @@ def test_batches_of_columns_and_other_grids(env, prec):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny,steps,seed", [(144, 100, 25, 7), (222, 175, 19, 33)])
+def test_coupled_adjoint_takes_the_fused_form_s_branches(env, nx, ny, steps, seed, monkeypatch):
+    """In the gas beside a solid phi = -(1 - phi0) to the last bit, where an ulp
+    decides whether the clamp of w passes a derivative.  The gradient on the node
+    step's states is that on the fused tile's (form 4): differences of rounding
+    alone are of order 1e-14, a branch taken otherwise is 1e-9 in d/dg_y."""
+    _, lbm = env
+    cfg, arr = W.sessile_droplet(nx, seed=seed, radius=0.2 * min(nx, ny), ny=ny)
+    grads = []
+    for form in ("0", "4"):
+        monkeypatch.setenv("LBM_KERNEL_FORM", form)
+        s = lbm.Solver(cfg, precision="fp64").set_geometry(arr)
+        grads.append(np.array(s.adjoint_coupled(steps, observable=0, every=16)[1]))
+        s.close()
+    a, b = grads
+    scale = np.abs(b).max()
+    assert np.all(np.abs(a - b) <= 1e-11 * np.abs(b) + 1e-13 * scale), (a, b)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny", [(70, 12), (40, 33)])
 def test_coupled_adjoint_runs_where_the_local_planes_do_not_fit(env, nx, ny, monkeypatch):
     """Memory for the states alone is enough: an allocation with room for their
