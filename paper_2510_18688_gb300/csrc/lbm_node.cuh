@@ -31,7 +31,7 @@
 // and differ only in where they store.
 //
 // Measured (GB300): the double 512 x 512 droplet with sums every step, 374 us
-// a step as one fused 32 x 8 tile kernel, 186 us as these two (36 + 150; 345
+// a step as one fused 32 x 8 tile kernel, 188 us as these two (35 + 153; 347
 // FP64 instructions a node against about 640 and the ring's; FP64 pipe 85 %
 // busy); the tangent step of 250 x 190 nodes 298 us and 88 us.
 #pragma once
@@ -904,7 +904,7 @@ __device__ __forceinline__ void node_collide(const NodeArgs<R, D>& a, const Read
           // tile.  In the gas beside a solid phi = -(1 - phi0) to the last bit, and
           // an ulp decides whether the clamp of w passes a derivative: with one
           // rounding fewer (phi 8 % nearer to an 80-bit solution, two
-          // instructions of 290 less) d/dg_y of sweeps under 30 steps is 1e-11 to
+          // instructions of 291 less) d/dg_y of sweeps under 30 steps is 1e-11 to
           // 2e-9 away from that form's.
           const R eq0 = mad(mul(mu, c.eta), k_t(L_::w0 - 1.0), phi);
           const R r0 = mad(gq[0], c.omg, mul_rn(eq0, c.itg));
